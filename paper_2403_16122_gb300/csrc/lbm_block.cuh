@@ -159,11 +159,10 @@ struct BlockPops {
     __device__ __forceinline__ float4 own0() const {
         return *reinterpret_cast<const float4*>(sl + BlockSlot<ST>::kOwn + 16 * lane);
     }
-    __device__ __forceinline__ float G(int i) const { return i == 0 ? own0().x : pair(i).x; }
-    __device__ __forceinline__ float H(int i) const {
-        if (i == 0) return own0().y;
-        const float v = pair(i).y;
-        return ((dmask >> i) & 1) ? -v + 2.0f * WGT(i) * abb : v;
+    __device__ __forceinline__ float2 GH(int i) const {
+        if (i == 0) return make_float2(own0().x, own0().y);
+        const float2 v = pair(i);
+        return make_float2(v.x, ((dmask >> i) & 1) ? -v.y + 2.0f * WGT(i) * abb : v.y);
     }
     __device__ __forceinline__ float F(int i) const { return f[i]; }
 };
@@ -251,7 +250,7 @@ __device__ __forceinline__ bool block_item(const Inst* __restrict__ insts, const
     const bool out_lane = lane < w;
     const ST* A = static_cast<const ST*>(I.pop[parity]);
     const float* Aaux = I.aux[parity];
-    const float abb = P.Cpref * P.Tw;
+    const float abb = P.abb();
     // side columns (periodic x)
     const int cL1 = wrapi(x0 - 1, nx), cL2 = wrapi(x0 - 2, nx);
     const int cR1 = wrapi(x0 + w, nx), cR2 = wrapi(x0 + w + 1, nx);
@@ -498,7 +497,7 @@ __device__ __forceinline__ bool block_item(const Inst* __restrict__ insts, const
         if (top_wall) {
             // row ny lies behind the top wall: ghost from rows ny-1 and ny-2
             php = wet_ghost(ph0, left(ph0, sPhi[0][1]), right(ph0, sPhi[1][1]),
-                            left(phm, sPhi[0][0]), right(phm, sPhi[1][0]), P.tan_w);
+                            left(phm, sPhi[0][0]), right(phm, sPhi[1][0]), P.rare->tan_w);
             rhp = rh0; pp = p0; Sp = S0; tp = t0;
 #pragma unroll
             for (int sd = 0; sd < 2; ++sd) {
@@ -508,21 +507,21 @@ __device__ __forceinline__ bool block_item(const Inst* __restrict__ insts, const
                 const float in2 = __shfl_sync(0xffffffffu, phm, sd == 0 ? 0 : w - 1);
                 const float out1 = hv(jy, sd, 5), out2 = hv(jy - 1, sd, 5);
                 // left side column: out is its left neighbour, in its right one
-                sPhi[sd][2] = sd == 0 ? wet_ghost(sPhi[sd][1], out1, in1, out2, in2, P.tan_w)
-                                      : wet_ghost(sPhi[sd][1], in1, out1, in2, out2, P.tan_w);
+                sPhi[sd][2] = sd == 0 ? wet_ghost(sPhi[sd][1], out1, in1, out2, in2, P.rare->tan_w)
+                                      : wet_ghost(sPhi[sd][1], in1, out1, in2, out2, P.rare->tan_w);
             }
         }
         if (bottom_wall) {
             phm = wet_ghost(ph0, left(ph0, sPhi[0][1]), right(ph0, sPhi[1][1]),
-                            left(php, sPhi[0][2]), right(php, sPhi[1][2]), P.tan_w);
+                            left(php, sPhi[0][2]), right(php, sPhi[1][2]), P.rare->tan_w);
             rhm = rh0; pm = p0; Sm = S0; tm = t0;
 #pragma unroll
             for (int sd = 0; sd < 2; ++sd) {
                 const float in1 = __shfl_sync(0xffffffffu, ph0, sd == 0 ? 0 : w - 1);
                 const float in2 = __shfl_sync(0xffffffffu, php, sd == 0 ? 0 : w - 1);
                 const float out1 = hv(jy, sd, 5), out2 = hv(jy + 1, sd, 5);
-                sPhi[sd][0] = sd == 0 ? wet_ghost(sPhi[sd][1], out1, in1, out2, in2, P.tan_w)
-                                      : wet_ghost(sPhi[sd][1], in1, out1, in2, out2, P.tan_w);
+                sPhi[sd][0] = sd == 0 ? wet_ghost(sPhi[sd][1], out1, in1, out2, in2, P.rare->tan_w)
+                                      : wet_ghost(sPhi[sd][1], in1, out1, in2, out2, P.rare->tan_w);
             }
         }
 

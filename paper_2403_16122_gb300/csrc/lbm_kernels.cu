@@ -214,25 +214,28 @@ __device__ __forceinline__ void pull_set(const LatT<NC>& l, int x, int y, float 
     }
 }
 
+// Physics constants that every site needs, in registers; those of options and
+// walls are read through `rare` where they are used (16 registers fewer across
+// the row loop of the strip kernels).
 struct Phys {
-    float L, Hs, Tm, Cp, Cpref, Tw, omega_g, omega_h, kappa, beta, lam_coef;
-    float rho_s, rho_l, rho_g, mu_s, mu_l, mu_g, mdot_coef, tan_w, inv_ramp, eps2;
+    float L, Hs, Tm, Cp, Cpref, omega_g, omega_h, kappa, beta, lam_coef;
+    float rho_s, rho_l, rho_g, mu_s, mu_l, mu_g, mdot_coef, inv_ramp, eps2;
     float inv_L, inv_Cp;
-    float buoy_x, buoy_y, T_ref;
-    float Cp_s, Cp_g, k_s, k_g, dtau_h;
+    const Inst* __restrict__ rare;  // T_w, tan_w, Boussinesq, per-phase properties
     bool phase_props;
+    // Cp_ref T_w of the anti-bounce-back at Dirichlet walls
+    __device__ __forceinline__ float abb() const { return Cpref * rare->Tw; }
 };
 
 __device__ __forceinline__ Phys load_phys(const Inst& I) {
     Phys P;
-    P.L = I.L; P.Hs = I.Hs; P.Tm = I.Tm; P.Cp = I.Cp; P.Cpref = I.Cpref; P.Tw = I.Tw;
+    P.L = I.L; P.Hs = I.Hs; P.Tm = I.Tm; P.Cp = I.Cp; P.Cpref = I.Cpref;
     P.omega_g = I.omega_g; P.omega_h = I.omega_h; P.kappa = I.kappa; P.beta = I.beta;
     P.lam_coef = I.lam_coef; P.rho_s = I.rho_s; P.rho_l = I.rho_l; P.rho_g = I.rho_g;
     P.mu_s = I.mu_s; P.mu_l = I.mu_l; P.mu_g = I.mu_g; P.mdot_coef = I.mdot_coef;
-    P.tan_w = I.tan_w; P.inv_ramp = I.inv_ramp; P.eps2 = I.normal_eps2;
+    P.inv_ramp = I.inv_ramp; P.eps2 = I.normal_eps2;
     P.inv_L = I.inv_L; P.inv_Cp = I.inv_Cp;
-    P.buoy_x = I.buoy_x; P.buoy_y = I.buoy_y; P.T_ref = I.T_ref;
-    P.Cp_s = I.Cp_s; P.Cp_g = I.Cp_g; P.k_s = I.k_s; P.k_g = I.k_g; P.dtau_h = I.dtau_h;
+    P.rare = &I;
     P.phase_props = (I.flags & kPhaseProps) != 0;
     return P;
 }
@@ -267,7 +270,7 @@ __device__ __forceinline__ Macro local_macro(const Phys& P, const float g[9], co
     // - f_l); inside the mushy range the exact value is T_m (evaluating the sum
     // there would only add the rounding of f_l times L)
     if (P.phase_props) {  // sensible branches with the local C_p of Eq. 1
-        const float cp = mix3(fs, phi, P.Cp_s, P.Cp, P.Cp_g);
+        const float cp = mix3(fs, phi, P.rare->Cp_s, P.Cp, P.rare->Cp_g);
         m.T = m.mushy ? P.Tm : P.Tm + (Hp - P.Hs + P.L * (flp - fl)) / cp;
     } else {
         m.T = m.mushy ? P.Tm : P.Tm + (Hp - P.Hs + P.L * (flp - fl)) * P.inv_Cp;
@@ -367,28 +370,28 @@ __device__ __forceinline__ float lap_cols(float cL, float cC, float cR, float sL
 
 // Pulled populations of one site as site_update reads them: from arrays, or
 // (row-staged FP32 strips) straight from the lane's ring slot at each use, so
-// that they need not stay live in registers across the collision. The slot
-// form applies the anti-bounce-back of h on the links in hmask.
+// that they need not stay live in registers across the collision: the (g_i,
+// h_i) pair by one 8-byte load.
 struct ArrPops {
     const float *g, *h, *f;
-    __device__ __forceinline__ float G(int i) const { return g[i]; }
-    __device__ __forceinline__ float H(int i) const { return h[i]; }
+    __device__ __forceinline__ float2 GH(int i) const { return make_float2(g[i], h[i]); }
     __device__ __forceinline__ float F(int i) const { return f[i]; }
 };
+// Volatile, so that the value is read here and not kept since an earlier read.
+__device__ __forceinline__ float2 ld_pair(const float* p) {
+    float2 v;
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
 struct SlotPops {
     const float* s;  // the slot (layout: see the row staging below)
     int lane;
-    int hmask;       // bit i: h_i arrives through a Dirichlet wall
-    float abb;       // Cp_ref T_w
     __device__ __forceinline__ float rd(int off) const {
         return *reinterpret_cast<const volatile float*>(s + off);
     }
-    __device__ __forceinline__ float G(int i) const {
-        return rd(i == 0 ? 4 * lane : 256 + 64 * (i - 1) + 2 * lane);
-    }
-    __device__ __forceinline__ float H(int i) const {
-        const float v = rd(i == 0 ? 4 * lane + 1 : 256 + 64 * (i - 1) + 2 * lane + 1);
-        return ((hmask >> i) & 1) ? -v + 2.0f * WGT(i) * abb : v;
+    __device__ __forceinline__ float2 GH(int i) const {
+        return ld_pair(s + (i == 0 ? 4 * lane : 256 + 64 * (i - 1) + 2 * lane));
     }
     __device__ __forceinline__ float F(int i) const {
         return rd(i == 0 ? 4 * lane + 2 : 768 + 32 * (i - 1) + lane);
@@ -401,14 +404,8 @@ struct SlotGHPops {
     const float* s;
     int lane;
     const float* f;
-    __device__ __forceinline__ float rd(int off) const {
-        return *reinterpret_cast<const volatile float*>(s + off);
-    }
-    __device__ __forceinline__ float G(int i) const {
-        return rd(i == 0 ? 4 * lane : 256 + 64 * (i - 1) + 2 * lane);
-    }
-    __device__ __forceinline__ float H(int i) const {
-        return rd(i == 0 ? 4 * lane + 1 : 256 + 64 * (i - 1) + 2 * lane + 1);
+    __device__ __forceinline__ float2 GH(int i) const {
+        return ld_pair(s + (i == 0 ? 4 * lane : 256 + 64 * (i - 1) + 2 * lane));
     }
     __device__ __forceinline__ float F(int i) const { return f[i]; }
 };
@@ -578,8 +575,8 @@ __device__ __forceinline__ void site_update_to(const Phys& P, int flags, const M
     float Fx = muphi * gphx, Fy = muphi * gphy;
     if (flags & kStMask) { Fx *= (1.f - fs); Fy *= (1.f - fs); }
     if (flags & kBuoy) {  // Boussinesq buoyancy of Section 4.3 at every site
-        Fx += P.buoy_x * (m.T - P.T_ref);
-        Fy += P.buoy_y * (m.T - P.T_ref);
+        Fx += P.rare->buoy_x * (m.T - P.rare->T_ref);
+        Fy += P.rare->buoy_y * (m.T - P.rare->T_ref);
     }
 
     // Eqs. 34-35: u* from the flow moments, solid forcing f = -f_s u*
@@ -632,13 +629,14 @@ __device__ __forceinline__ void site_update_to(const Phys& P, int flags, const M
     // per-phase properties: local C_p in h^eq, tau_h - 1/2 scaled by k / k_l
     float Cp_loc = P.Cp, omega_h = P.omega_h;
     if (P.phase_props) {
-        Cp_loc = mix3(fs, phi, P.Cp_s, P.Cp, P.Cp_g);
-        omega_h = 1.f / (mix3(fs, phi, P.k_s, 1.f, P.k_g) * P.dtau_h + 0.5f);
+        Cp_loc = mix3(fs, phi, P.rare->Cp_s, P.Cp, P.rare->Cp_g);
+        omega_h = 1.f / (mix3(fs, phi, P.rare->k_s, 1.f, P.rare->k_g) * P.rare->dtau_h + 0.5f);
     }
     const float TCp = T * Cp_loc, TCpref = T * P.Cpref;
     const float uu15 = 1.5f * uu;
     // rest populations (c_0 = 0)
-    const float gi0 = pop.G(0), hi0 = pop.H(0), fi0 = pop.F(0);
+    const float2 gh0 = pop.GH(0);
+    const float gi0 = gh0.x, hi0 = gh0.y, fi0 = pop.F(0);
     float g0n, h0n, f0n;
     {
         const float si = kW0 * -uu15;
@@ -685,11 +683,12 @@ __device__ __forceinline__ void site_update_to(const Phys& P, int flags, const M
         // g (Eqs. 21, 24, 25)
         const float2 geq = __ffma2_rn(bc(phi * w3cu), sgn, bc(w * phi));
         const float2 Gi = __ffma2_rn(bc(3.f * w * cdot(i, ax, ay)), sgn, bc(w * pmd));
-        const float2 g = make_float2(pop.G(i), pop.G(j));
+        const float2 ghi = pop.GH(i), ghj = pop.GH(j);
+        const float2 g = make_float2(ghi.x, ghj.x);
         const float2 gn = __ffma2_rn(bc(gsrc), Gi, __ffma2_rn(og, sub2(g, geq), g));
         // h (Eqs. 27-28)
         const float2 heq = __ffma2_rn(bc(TCp), si, bc(w * TCpref));
-        const float2 h = make_float2(pop.H(i), pop.H(j));
+        const float2 h = make_float2(ghi.y, ghj.y);
         const float2 hn = __ffma2_rn(oh, sub2(h, heq), h);
         if constexpr (sizeof(ST) == 4) {
             out.gh32(i, gn.x, hn.x);
@@ -779,7 +778,7 @@ __device__ __forceinline__ void tile_step(const Inst& I, const Tile& T, int pari
     l.plane = (int)I.plane; l.nx = I.nx; l.ny = I.ny; l.pitch = I.pitch; l.flags = I.flags;
     float* __restrict__ B = static_cast<float*>(I.pop[parity ^ 1]);
     float* __restrict__ Baux = I.aux[parity ^ 1];
-    const float abb = P.Cpref * P.Tw;
+    const float abb = P.abb();
 
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
@@ -908,14 +907,14 @@ __device__ __forceinline__ void tile_step(const Inst& I, const Tile& T, int pari
             const int xm = wrap_or_clamp(gx - 1, l.nx, px), xp = wrap_or_clamp(gx + 1, l.nx, px);
             const float d0 = 0.5f * (s_phi[lat_slot(xp, ya)] - s_phi[lat_slot(xm, ya)]);
             const float d1 = 0.5f * (s_phi[lat_slot(xp, yb)] - s_phi[lat_slot(xm, yb)]);
-            ghost = s_phi[lat_slot(gx, ya)] + P.tan_w * fabsf(1.5f * d0 - 0.5f * d1);
+            ghost = s_phi[lat_slot(gx, ya)] + P.rare->tan_w * fabsf(1.5f * d0 - 0.5f * d1);
         } else if (outx && !outy) {
             const int xa = cxl, xb = (x0 + ox < 0) ? 1 : l.nx - 2;
             const bool py = (l.flags & kPeriodicY) != 0;
             const int ym = wrap_or_clamp(gy - 1, l.ny, py), yp = wrap_or_clamp(gy + 1, l.ny, py);
             const float d0 = 0.5f * (s_phi[lat_slot(xa, yp)] - s_phi[lat_slot(xa, ym)]);
             const float d1 = 0.5f * (s_phi[lat_slot(xb, yp)] - s_phi[lat_slot(xb, ym)]);
-            ghost = s_phi[lat_slot(xa, gy)] + P.tan_w * fabsf(1.5f * d0 - 0.5f * d1);
+            ghost = s_phi[lat_slot(xa, gy)] + P.rare->tan_w * fabsf(1.5f * d0 - 0.5f * d1);
         } else {
             ghost = s_phi[lat_slot(cxl, cyl)];
         }
@@ -998,7 +997,7 @@ step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int pa
 // observable partials go to the caller-supplied scratch array.
 template <bool OBS>
 __global__ void __launch_bounds__(256)
-step_tile_noalloc(const Inst I, int tiles_x, double* __restrict__ partials) {
+step_tile_noalloc(const __grid_constant__ Inst I, int tiles_x, double* __restrict__ partials) {
     Tile T;
     T.inst = 0;
     T.x0 = (int)(blockIdx.x % tiles_x) * 32;
@@ -1198,17 +1197,21 @@ __device__ __forceinline__ void stage_row(const LatT<NC>& l, int lane, const Col
     cp_async_cg16(slot + kSlotO1 + 4 * lane, l.Aaux + ra + ct.aux + 128, pol);
     if constexpr (kHalf) cp_async_p<8>(slot + kSlotR + 2 * lane, l.Aaux + ra + ct.ref, pol);
     const unsigned short* A16 = reinterpret_cast<const unsigned short*>(l.A);
+    // The element a direction's values come from is row term + column term +
+    // place in the chunk. Chunks P and M list opposite directions in the same
+    // order, so a bounced direction keeps its place and only the terms change:
+    // the opposite chunk of the row itself and the lane's own column. They are
+    // chosen once per chunk, not per direction.
+    const int rP = wlo ? t0 + kChunkM : tm + kChunkP, rM = whi ? t0 + kChunkP : tp + kChunkM;
+    const int rZ = t0 + kChunkZ;
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
         const int cy = CY(i), cx = CX(i);
-        const bool wall = (cy > 0 && wlo) || (cy < 0 && whi);
-        const int si = wall ? OPP(i) : i;
-        // source: the site itself (bounce-back) or x - c_i in row y - c_iy
-        // (the column index is a constant: no array indexed at run time)
-        const int k = cx > 0 ? 0 : (cx < 0 ? 2 : 1);
-        const int rt = wall ? t0 : (cy > 0 ? tm : (cy < 0 ? tp : t0));
-        const int cg = wall ? ct.gh[1] : ct.gh[k], cf = wall ? ct.f[1] : ct.f[k];
-        const int eg = rt + cg + gh_off(si), ef = rt + cf + f_off(si);
+        const int k = cx > 0 ? 0 : (cx < 0 ? 2 : 1);  // column x - c_i
+        const bool wall = cy > 0 ? wlo : (cy < 0 ? whi : false);
+        const int rt = cy > 0 ? rP : (cy < 0 ? rM : rZ);
+        const int cg = k != 1 && wall ? ct.gh[1] : ct.gh[k], cf = k != 1 && wall ? ct.f[1] : ct.f[k];
+        const int eg = rt + cg + 64 * chunk_k(i), ef = rt + cf + 64 * chunk_n(i) + 32 * chunk_k(i);
         if constexpr (kHalf) {
             // blocks and plane rows hold an even number of 16-bit values, so
             // every aligned word lies inside its plane row
@@ -1231,67 +1234,58 @@ struct ColPar {
 };
 __device__ __forceinline__ unsigned half_sel(int col) { return (col & 1) ? 0x3232u : 0x1010u; }
 
-// Set `set` of a staged row, decoded as pull_set does: for FP16 storage with
-// the site's own references (g, h) and the source pressures pref (f; the
-// site's own pressure pref[0] on bounced links); for h at a Dirichlet wall
-// row the bounced populations become anti-bounce-back, -h + 2 w_i Cp_ref T_w.
-template <int SET, typename ST = float>
-__device__ __forceinline__ void staged_set(const float* slot, int lane, int r, int ny, bool py,
-                                           int flags, float abb, float v[9],
-                                           const ColPar& par = ColPar{0, 0, 0},
-                                           const Ref& ref = Ref{0.f, 0.f}, float Cpref = 0.f,
-                                           const float* pref = nullptr) {
-    const bool wlo = !py && r == 0, whi = !py && r == ny - 1;
-    v[0] = slot[4 * lane + SET];  // FP32 rest population (h_0 shifted)
-    if constexpr (sizeof(ST) == 4) {
-#pragma unroll
-        for (int i = 1; i < 9; ++i) v[i] = SET < 2 ? slot[slot_gh(i, lane) + SET] : slot[slot_f(i, lane)];
-        if (SET == 1 && !py) {
-            const bool lo = wlo && (flags & kDirYlo), hi = whi && (flags & kDirYhi);
-#pragma unroll
-            for (int i = 1; i < 9; ++i)
-                if ((CY(i) > 0 && lo) || (CY(i) < 0 && hi)) v[i] = -v[i] + 2.0f * WGT(i) * abb;
-        }
-    } else {
+// g and h of a staged row: each (g_i, h_i) pair read once. 16-bit storage
+// decodes it with the site's own references. In a row at a Dirichlet wall the
+// bounced h become anti-bounce-back, -h + 2 w_i Cp_ref T_w, and go back into
+// the slot, as every decoded pair of 16-bit storage does: the collision then
+// reads the slot as it is, without a select per direction. Only wall rows pay.
+template <typename ST>
+__device__ __forceinline__ void staged_gh(float* slot, int lane, bool dlo, bool dhi, const Phys& P,
+                                          float g[9], float h[9], const Ref& ref) {
+    const float Cpref = P.Cpref;
+    const float2 r0 = *reinterpret_cast<const float2*>(slot + 4 * lane);  // h_0 shifted
+    g[0] = r0.x;
+    h[0] = r0.y;
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
-        const bool wall = (CY(i) > 0 && wlo) || (CY(i) < 0 && whi);
-        if (SET < 2) {
-            const unsigned w = __float_as_uint(slot[slot_gh(i, lane)]);
-            const float raw = Bits16<ST>::to_f(
-                Bits16<ST>::from_bits((unsigned short)(SET == 0 ? (w & 0xffffu) : (w >> 16))));
-            v[i] = SET == 0 ? raw + WGT(i) * ref.phi : raw + WGT(i) * Cpref * ref.T;
+        if constexpr (sizeof(ST) == 4) {
+            const float2 v = *reinterpret_cast<const float2*>(slot + slot_gh(i, lane));
+            g[i] = v.x;
+            h[i] = v.y;
         } else {
-            const unsigned w = __float_as_uint(slot[slot_f(i, lane)]);
-            const unsigned sel = wall ? par.c : (CX(i) > 0 ? par.m : (CX(i) < 0 ? par.p : par.c));
-            v[i] = Bits16<ST>::fma_lo_2m12(__byte_perm(w, 0u, sel), f_rest(i, wall ? pref[0] : pref[i]));
-        }
-        if (SET == 1 && wall) {
-            const bool dir = (wlo && (flags & kDirYlo)) || (whi && (flags & kDirYhi));
-            if (dir) v[i] = -v[i] + 2.0f * WGT(i) * abb;
+            const unsigned wd = __float_as_uint(slot[slot_gh(i, lane)]);
+            g[i] = Bits16<ST>::add_lo(wd, WGT(i) * ref.phi);
+            h[i] = Bits16<ST>::add_hi(wd, WGT(i) * Cpref * ref.T);
         }
     }
+    if (dlo || dhi) {
+        const float abb = P.abb();
+#pragma unroll
+        for (int i = 1; i < 9; ++i)
+            if (CY(i) != 0 && (CY(i) > 0 ? dlo : dhi)) {
+                h[i] = -h[i] + 2.0f * WGT(i) * abb;
+                if constexpr (sizeof(ST) == 4) slot[slot_gh(i, lane) + 1] = h[i];
+            }
+    }
+    if constexpr (sizeof(ST) != 4) {
+#pragma unroll
+        for (int i = 1; i < 9; ++i)
+            *reinterpret_cast<float2*>(slot + slot_gh(i, lane)) = make_float2(g[i], h[i]);
     }
 }
 
-// Sets g and h of a staged row together (16-bit storage): each (g_i, h_i)
-// word is loaded once and decoded by one paired conversion, then treated as
-// staged_set treats it.
+// f of a staged row of 16-bit storage, decoded with the source pressures pref
+// (the site's own pressure pref[0] on links that bounce at a wall).
 template <typename ST>
-__device__ __forceinline__ void staged_gh(const float* slot, int lane, int r, int ny, bool py,
-                                          int flags, float abb, float g[9], float h[9],
-                                          const Ref& ref, float Cpref) {
-    const bool wlo = !py && r == 0, whi = !py && r == ny - 1;
-    const bool dir = (wlo && (flags & kDirYlo)) || (whi && (flags & kDirYhi));
-    g[0] = slot[4 * lane];
-    h[0] = slot[4 * lane + 1];
+__device__ __forceinline__ void staged_f16(const float* slot, int lane, bool wlo, bool whi,
+                                           float v[9], const ColPar& par, const float* pref) {
+    v[0] = slot[4 * lane + 2];  // FP32 rest population
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
-        const unsigned wd = __float_as_uint(slot[slot_gh(i, lane)]);
-        g[i] = Bits16<ST>::add_lo(wd, WGT(i) * ref.phi);
-        h[i] = Bits16<ST>::add_hi(wd, WGT(i) * Cpref * ref.T);
         const bool wall = (CY(i) > 0 && wlo) || (CY(i) < 0 && whi);
-        if (wall && dir) h[i] = -h[i] + 2.0f * WGT(i) * abb;
+        const unsigned w = __float_as_uint(slot[slot_f(i, lane)]);
+        const unsigned sel = wall ? par.c : (CX(i) > 0 ? par.m : (CX(i) < 0 ? par.p : par.c));
+        v[i] = Bits16<ST>::fma_lo_2m12(__byte_perm(w, 0u, sel), f_rest(i, wall ? pref[0] : pref[i]));
     }
 }
 
@@ -1317,7 +1311,7 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     l.plane = (int)I.plane; l.nx = I.nx; l.ny = I.ny; l.pitch = I.pitch; l.flags = I.flags;
     void* __restrict__ B = I.pop[parity ^ 1];
     float* __restrict__ Baux = I.aux[parity ^ 1];
-    const float abb = P.Cpref * P.Tw;
+    const float abb = P.abb();
     const int nx = l.nx, ny = l.ny;
 
     RowCtx c;
@@ -1348,12 +1342,22 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         pull_set<1, ST>(l, x_outer, y, abb, hh, r, P.Cpref);
         return local_macro(P, gg, hh, ldAux(l, 0, idx)).phi;
     };
-    auto note_outer = [&](int y) {
+    // Only an item at a wall needs them, once: one copy of the pull code, in a
+    // loop that is not unrolled. (Computed inside the row step, where each row
+    // is first seen, it was instantiated four times at each of three places:
+    // 7,200 of the kernel's 9,312 instructions, and the step's second stall was
+    // the instruction fetch.)
+    auto note_outer = [&]() {
         if (c.py || !halo_lane) return;
-        if (y == 0) oB0 = outer_phi(y);
-        if (y == 1) oB1 = outer_phi(y);
-        if (y == ny - 1) oT0 = outer_phi(y);
-        if (y == ny - 2) oT1 = outer_phi(y);
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            if (k < 2 ? W.y0 != 0 : W.y1 != ny) continue;
+            const float v = outer_phi(k < 2 ? k : ny + 1 - k);
+            if (k == 0) oB0 = v;
+            else if (k == 1) oB1 = v;
+            else if (k == 2) oT0 = v;
+            else oT1 = v;
+        }
     };
     // local macroscopic fields of row y at this lane's column (the pulled g
     // and h are dropped; the collision of the row pulls them again, from L1)
@@ -1366,19 +1370,18 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         m = local_macro(P, gg, hh, ldAux(l, 0, idx));
         p = ldAux(l, 3, idx);
         S = ldAux(l, 4, idx);
-        note_outer(y);
     };
 
     // staged rows: ring index j <-> lattice row y0 - 1 + j, j = 0 .. R - 1
     const int y0 = W.y0;
     const int R = W.y1 - y0 + 2;
     const bool has_lo = y0 >= 1 || c.py, has_hi = W.y1 < ny || c.py;
-    auto slot = [&](int j) { return ring + (j % (STG > 0 ? STG : 1)) * slot_floats<ST>(); };
-    auto issue = [&](int j) {
+    auto slot = [&](int q) { return ring + q * slot_floats<ST>(); };  // ring place q < STG
+    auto issue = [&](int j, int q) {  // ring index j into place q = j mod STG
         if constexpr (STG > 0) {
             if (j < R && (j > 0 || has_lo) && (j < R - 1 || has_hi))
                 stage_row<ST>(l, lane, ct, c.py, y0 - 1 + j, j == 0 || j == R - 1,
-                              slot(j), j <= 1 ? 1 : (j >= R - 2 ? 2 : 0));
+                              slot(q), j <= 1 ? 1 : (j >= R - 2 ? 2 : 0));
             cp_async_commit();  // possibly empty: one group per ring index
         }
     };
@@ -1388,24 +1391,16 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         if constexpr (kHalf) { r.phi = sl[kSlotR + 2 * lane]; r.T = sl[kSlotR + 2 * lane + 1]; }
         return r;
     };
-    auto row_macro_staged = [&](int j, int y, Macro& m, float& p, float& S, Ref& r) {
+    const bool wy = !c.py;
+    auto row_macro_staged = [&](float* sl, int y, Macro& m, float& p, float& S, Ref& r) {
         float gg[9], hh[9];
-        const float* sl = slot(j);
         r = slot_ref(sl);
-        if constexpr (kHalf) {
-            staged_gh<ST>(sl, lane, y, ny, c.py, l.flags, abb, gg, hh, r, P.Cpref);
-            float* ws = const_cast<float*>(sl);  // the decoded values, for the collision
-#pragma unroll
-            for (int i = 1; i < 9; ++i)
-                *reinterpret_cast<float2*>(ws + slot_gh(i, lane)) = make_float2(gg[i], hh[i]);
-        } else {
-            staged_set<0, ST>(sl, lane, y, ny, c.py, l.flags, abb, gg, par, r, P.Cpref);
-            staged_set<1, ST>(sl, lane, y, ny, c.py, l.flags, abb, hh, par, r, P.Cpref);
-        }
+        staged_gh<ST>(sl, lane, wy && y == 0 && (l.flags & kDirYlo),
+                      wy && y == ny - 1 && (l.flags & kDirYhi), P, gg, hh, r);
         m = local_macro(P, gg, hh, sl[4 * lane + 3]);
-        p = sl[kSlotO1 + 4 * lane + 2];
-        S = sl[kSlotO1 + 4 * lane + 3];
-        note_outer(y);
+        const float2 ps = *reinterpret_cast<const float2*>(sl + kSlotO1 + 4 * lane + 2);
+        p = ps.x;
+        S = ps.y;
     };
 
     RowObs ob;
@@ -1425,26 +1420,30 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     Ref rO;
     if constexpr (STG > 0) {
 #pragma unroll 1
-        for (int j = 0; j < STG; ++j) issue(j);  // one copy of the row issue code
+        for (int j = 0; j < STG; ++j) issue(j, j);  // one copy of the row issue code
+        note_outer();              // while the copies are in flight
         cp_async_wait<STG - 2>();  // ring indices 0 and 1 have landed
-        row_macro_staged(1, y0, mO, p0, S0, rO);
+        row_macro_staged(slot(1), y0, mO, p0, S0, rO);
     } else {
+        note_outer();
         row_macro(y0, mO, p0, S0, rO);
     }
     ph0 = mO.phi; rh0 = mO.rho; t0 = mO.T;
     if (has_lo) {
         Macro mm;
         Ref rr;
-        if constexpr (STG > 0) row_macro_staged(0, y0 == 0 ? ny - 1 : y0 - 1, mm, pm, Sm, rr);
+        if constexpr (STG > 0) row_macro_staged(slot(0), y0 == 0 ? ny - 1 : y0 - 1, mm, pm, Sm, rr);
         else row_macro(y0 == 0 ? ny - 1 : y0 - 1, mm, pm, Sm, rr);
         phm = mm.phi; rhm = mm.rho; tm = mm.T;
     }
 
     for (int y = y0; y < W.y1; ++y) {
         const int own = y * l.pitch + c.xc;
-        const int jy = y - y0 + 1;  // ring index of row y
+        // ring places of rows y and y + 1
+        constexpr int RS = STG > 0 ? STG : 1;
+        const int qy = (y - y0 + 1) % RS, qn = (y - y0 + 2) % RS;
         if constexpr (STG > 0) {
-            issue(jy + STG - 1);        // into the slot of row y - 1, no longer read
+            issue(y - y0 + STG, (y - y0) % RS);  // into the slot of row y - 1, no longer read
             cp_async_wait<STG - 2>();   // row y + 1 has landed
         }
         // Every load that goes to DRAM for this row is issued here, before any
@@ -1466,18 +1465,16 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
                     pref[i] = lane_shift(v, -CX(i));                     // source column x - cx
                 }
             }
-            if constexpr (STG > 0)
-                staged_set<2, ST>(slot(jy), lane, y, ny, c.py, l.flags, abb, f, par, rO, P.Cpref,
-                                  pref);
+            if constexpr (STG > 0 && kHalf)
+                staged_f16<ST>(slot(qy), lane, wy && y == 0, wy && y == ny - 1, f, par, pref);
             else
                 pull_row<2, ST>(l, c, y, abb, f, rO, P.Cpref, pref);
         };
         float phiux_p, phiuy_p;
         if constexpr (STG > 0) {
-            const float* sl = slot(jy);
-            if constexpr (!kHalf && !kSlotPops) pull_f();
-            phiux_p = sl[kSlotO1 + 4 * lane];
-            phiuy_p = sl[kSlotO1 + 4 * lane + 1];
+            const float2 pu = *reinterpret_cast<const float2*>(slot(qy) + kSlotO1 + 4 * lane);
+            phiux_p = pu.x;
+            phiuy_p = pu.y;
         } else {
             if constexpr (!kHalf) pull_f();
             phiux_p = ldAux(l, 1, own);
@@ -1487,18 +1484,18 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         Ref rN{0.f, 0.f};
         const bool top_wall = !(y + 1 < ny || c.py);
         if (!top_wall) {
-            if constexpr (STG > 0) row_macro_staged(jy + 1, y + 1 == ny ? 0 : y + 1, mN, pp, Sp, rN);
+            if constexpr (STG > 0) row_macro_staged(slot(qn), y + 1 == ny ? 0 : y + 1, mN, pp, Sp, rN);
             else row_macro(y + 1 == ny ? 0 : y + 1, mN, pp, Sp, rN);
             php = mN.phi; rhp = mN.rho; tp = mN.T;
         } else {
             // row ny lies behind the top wall: ghost from rows ny-1 and ny-2
-            php = strip_wet_ghost(ph0, phm, oT0, oT1, lane, P.tan_w);
+            php = strip_wet_ghost(ph0, phm, oT0, oT1, lane, P.rare->tan_w);
             rhp = rh0; pp = p0; Sp = S0; tp = t0;
         }
         const bool bottom_wall = y == 0 && !c.py;
         if (bottom_wall) {
             // row -1 lies behind the bottom wall: ghost from rows 0 and 1
-            phm = strip_wet_ghost(ph0, php, oB0, oB1, lane, P.tan_w);
+            phm = strip_wet_ghost(ph0, php, oB0, oB1, lane, P.rare->tan_w);
             rhm = rh0; pm = p0; Sm = S0; tm = t0;
         }
         if constexpr (kHalf && STG == 0) pull_f();
@@ -1546,32 +1543,20 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         if constexpr (kSlotPops && kHalf) {
             pull_f();  // all lanes (shuffles); f stays in registers for the collision
             if (out_lane)
-                site_update<OBS, ST>(P, l.flags, mO, SlotGHPops{slot(jy), lane, f}, phiux_p,
+                site_update<OBS, ST>(P, l.flags, mO, SlotGHPops{slot(qy), lane, f}, phiux_p,
                                      phiuy_p, st, B, Baux, l.plane, own, c.xc == nx / 2,
                                      y == ny / 2, ob, dref);
         } else if constexpr (kSlotPops) {
             if (out_lane) {
-                int hmask = 0;
-                if (!kHalf && !c.py) {
-                    const bool lo = y == 0 && (l.flags & kDirYlo), hi = y == ny - 1 && (l.flags & kDirYhi);
-#pragma unroll
-                    for (int i = 1; i < 9; ++i)
-                        if ((CY(i) > 0 && lo) || (CY(i) < 0 && hi)) hmask |= 1 << i;
-                }
-                site_update<OBS, ST>(P, l.flags, mO, SlotPops{slot(jy), lane, hmask, abb}, phiux_p,
+                site_update<OBS, ST>(P, l.flags, mO, SlotPops{slot(qy), lane}, phiux_p,
                                      phiuy_p, st, B, Baux, l.plane, own, c.xc == nx / 2,
                                      y == ny / 2, ob, dref);
             }
         } else if (out_lane) {
             // g and h of row y were pulled one row earlier: these loads hit L1
             float g[9], h[9];
-            if constexpr (STG > 0) {
-                staged_set<0, ST>(slot(jy), lane, y, ny, c.py, l.flags, abb, g, par, rO, P.Cpref);
-                staged_set<1, ST>(slot(jy), lane, y, ny, c.py, l.flags, abb, h, par, rO, P.Cpref);
-            } else {
-                pull_row<0, ST>(l, c, y, abb, g, rO, P.Cpref);
-                pull_row<1, ST>(l, c, y, abb, h, rO, P.Cpref);
-            }
+            pull_row<0, ST>(l, c, y, abb, g, rO, P.Cpref);
+            pull_row<1, ST>(l, c, y, abb, h, rO, P.Cpref);
             site_update<OBS, ST>(P, l.flags, mO, ArrPops{g, h, f}, phiux_p, phiuy_p, st, B, Baux,
                                  l.plane, own, c.xc == nx / 2, y == ny / 2, ob, dref);
         }

@@ -99,6 +99,10 @@ int max_tiles_of(const lbm_params& p) {
     return ((p.nx + 31) / 32) * ((p.ny + 3) / 4);
 }
 
+// Default tile. Against 32 x 8 the shorter block spreads a small lattice over
+// twice the SMs: 2.7 us against 3.2 us a step on 256 x 8 sites, 3.6 against 4.1
+// on 203 x 151, 13.8 against 14.7 on 500 x 500.
+constexpr int kTileX = 32, kTileY = 4;
 constexpr int kMinRows = 2;  // shortest strip segment
 int max_items_of(const lbm_params& p) {
     return ((p.nx + lbmk::kStripW - 1) / lbmk::kStripW) * ((p.ny + kMinRows - 1) / kMinRows);
@@ -159,7 +163,9 @@ struct lbm_handle {
     int n_inst = 0;
     int storage = 0;
     int kind = LBM_KERNEL_TILE;
-    int tx = 32, ty = 8;                 // tile shape
+    int tx = kTileX, ty = kTileY;        // tile shape
+    bool chosen = true;                  // the layout is still the one lbm_create chose
+    bool small = false;                  // all lattices together: two waves of tiles at most
     int warps = 4, rows = 16, regs = 168; // strip layouts (rows: effective)
     int rows_req = 16;                    // requested rows per item, 0 = one wave
     std::vector<Item> items;
@@ -259,6 +265,20 @@ void build_tiles(lbm_handle* h) {
 bool is_strip(int kind) {
     return kind == LBM_KERNEL_STRIP || kind == LBM_KERNEL_STAGED || kind == LBM_KERNEL_BLOCK;
 }
+// Whether the steps of a handle run in tiles: the tile layout, or the layout
+// lbm_create chose for lattices that are at most two waves of tile CTAs (one
+// thread per site; 155,648 sites on 152 SMs). There a step is one chain of
+// latencies, and a strip item's is some rows longer than a tile's: 2.7 us
+// against 8.1 us a step on 128 x 96 sites, 4.1 against 8.3 on 256 x 256, 6.8
+// against 9.0 on 320 x 320. Beyond, the strips come level: 9.6 against 11.5 on
+// 400 x 400 but 26.4 against 24.3 for a step with its observables, 13.4 against
+// 14.6 on 512 x 512, 23.3 against 18.1 on 620 x 620. The persistent form stays
+// with the strips.
+bool tiled(const lbm_handle* h) {
+    return h->kind == LBM_KERNEL_TILE ||
+           (h->chosen && h->small && h->exec != LBM_EXEC_PERSISTENT);
+}
+
 // Output columns of one item of a strip-like layout.
 int item_width(int kind) { return kind == LBM_KERNEL_BLOCK ? lbmk::kBlockW : lbmk::kStripW; }
 
@@ -284,7 +304,6 @@ int item_rows(const lbm_handle* h) {
 
 void build_items(lbm_handle* h) {
     h->items.clear();
-    h->rows = item_rows(h);
     for (int k = 0; k < h->n_inst; ++k) {
         const lbm_params& p = h->params[k];
         h->inst[k].part_begin = (int)h->items.size();
@@ -301,6 +320,14 @@ void build_items(lbm_handle* h) {
             }
         h->inst[k].part_end = (int)h->items.size();
     }
+}
+
+int count_items(const lbm_handle* h) {
+    const int wd = item_width(h->kind);
+    int n = 0;
+    for (const auto& p : h->params)
+        n += ((p.nx + wd - 1) / wd) * ((p.ny + h->rows - 1) / h->rows);
+    return n;
 }
 
 void drop_graphs(lbm_handle* h) {
@@ -369,7 +396,8 @@ int upload_tables(lbm_handle* h) {
         cudaError_t e = lbmk::prepare_block(h->warps, h->regs, h->storage);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    if (is_strip(h->kind)) build_items(h); else build_tiles(h);
+    if (is_strip(h->kind)) h->rows = item_rows(h);
+    if (tiled(h)) build_tiles(h); else build_items(h);
     h->max_lattice_parts = 0;
     for (int k = 0; k < h->n_inst; ++k)
         h->max_lattice_parts =
@@ -377,7 +405,7 @@ int upload_tables(lbm_handle* h) {
     cudaError_t e = cudaMemcpyAsync(h->d_inst, h->inst.data(), sizeof(Inst) * h->n_inst,
                                     cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) return cuda_fail(e);
-    if (is_strip(h->kind))
+    if (!tiled(h))
         e = cudaMemcpyAsync(h->d_items, h->items.data(), sizeof(Item) * h->items.size(),
                             cudaMemcpyHostToDevice, h->stream);
     else
@@ -388,16 +416,19 @@ int upload_tables(lbm_handle* h) {
     if (e != cudaSuccess) return cuda_fail(e);
     h->persist_grid = h->kind == LBM_KERNEL_BLOCK
                           ? lbmk::block_persistent_grid(h->warps, h->regs, h->storage,
-                                                        (int)h->items.size())
+                                                        count_items(h))
                           : (is_strip(h->kind)
                                  ? lbmk::persistent_grid(h->kind == LBM_KERNEL_STAGED, h->warps,
-                                                         h->regs, h->storage, (int)h->items.size())
+                                                         h->regs, h->storage, count_items(h))
                                  : 0);
     return LBM_OK;
 }
 
 // One time step through the ordinary kernels (obs != 0: with observable partials).
 cudaError_t enqueue_step(lbm_handle* h, int parity, int obs, cudaStream_t s) {
+    if (tiled(h))
+        return lbmk::launch_step(h->tx, h->ty, h->storage, h->d_inst, h->d_tiles,
+                                 (int)h->tiles.size(), parity, obs, h->d_part, s);
     if (h->kind == LBM_KERNEL_BLOCK)
         return lbmk::launch_step_block(h->warps, h->regs, h->storage, h->d_inst, h->d_items,
                                        (int)h->items.size(), parity, obs, h->d_part,
@@ -405,11 +436,8 @@ cudaError_t enqueue_step(lbm_handle* h, int parity, int obs, cudaStream_t s) {
     if (h->kind == LBM_KERNEL_STAGED)
         return lbmk::launch_step_staged(h->warps, h->regs, h->storage, h->d_inst, h->d_items,
                                         (int)h->items.size(), parity, obs, h->d_part, s);
-    return h->kind == LBM_KERNEL_STRIP
-               ? lbmk::launch_step_strip(h->warps, h->regs, h->storage, h->d_inst, h->d_items,
-                                         (int)h->items.size(), parity, obs, h->d_part, s)
-               : lbmk::launch_step(h->tx, h->ty, h->storage, h->d_inst, h->d_tiles,
-                                   (int)h->tiles.size(), parity, obs, h->d_part, s);
+    return lbmk::launch_step_strip(h->warps, h->regs, h->storage, h->d_inst, h->d_items,
+                                   (int)h->items.size(), parity, obs, h->d_part, s);
 }
 
 // n steps without observables from `parity` as one persistent launch.
@@ -576,9 +604,15 @@ int lbm_create(const lbm_params* p, int32_t n_inst, int32_t storage, void* d_wor
     for (int k = 0; k < n_inst; ++k) fill_inst(h, k);
     bool all_px = true;
     for (int k = 0; k < n_inst; ++k) all_px = all_px && p[k].periodic_x;
-    // row-staged strips, one wave of items
+    // row-staged strips, one wave of items; small lattices run in tiles
     h->kind = all_px ? LBM_KERNEL_STAGED : LBM_KERNEL_TILE;
     h->rows_req = 0;
+    if (storage == LBM_STORE_FP32) {
+        long long n_tiles = 0;
+        for (int k = 0; k < n_inst; ++k)
+            n_tiles += (long long)((p[k].nx + kTileX - 1) / kTileX) * ((p[k].ny + kTileY - 1) / kTileY);
+        h->small = n_tiles <= 2 * lbmk::tile_resident_ctas(kTileX, kTileY);
+    }
     rc = upload_tables(h);
     if (rc != LBM_OK) {
         delete h;
@@ -992,6 +1026,7 @@ int lbm_set_kernel(lbm_handle* h, int32_t kind, int32_t a, int32_t b, int32_t c)
     } else {
         return LBM_EINVAL;
     }
+    h->chosen = false;
     h->have_obs = false;  // partial slots are renumbered
     return upload_tables(h);
 }
@@ -1003,9 +1038,10 @@ int lbm_set_exec(lbm_handle* h, int32_t mode, int32_t chunk) {
     if (mode == LBM_EXEC_PERSISTENT && (!is_strip(h->kind) || h->persist_grid <= 0))
         return LBM_EINVAL;
     drop_graphs(h);
+    const bool was_tiled = tiled(h);
     h->exec = mode;
     h->chunk = chunk;
-    return LBM_OK;
+    return tiled(h) == was_tiled ? LBM_OK : upload_tables(h);
 }
 
 int lbm_get_exec(const lbm_handle* h, int32_t* out) {
@@ -1059,6 +1095,7 @@ int lbm_autotune(lbm_handle* h, int32_t steps, double* times_ms, int32_t cap, in
             for (auto& v : bvar) cands.push_back({LBM_KERNEL_BLOCK, v[0], r, v[1]});
     }
     if (h->exec != LBM_EXEC_PERSISTENT) {  // the persistent form is strip-only
+        cands.push_back({LBM_KERNEL_TILE, 32, 4, 0});
         cands.push_back({LBM_KERNEL_TILE, 32, 8, 0});
         cands.push_back({LBM_KERNEL_TILE, 64, 4, 0});
         cands.push_back({LBM_KERNEL_TILE, 32, 16, 0});

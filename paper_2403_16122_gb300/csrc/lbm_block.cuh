@@ -122,9 +122,7 @@ __device__ __forceinline__ int dir_shift(int i, const RowSrc& r) { return dir_bo
 // next one b, given each one's neighbours on both sides.
 __device__ __forceinline__ float wet_ghost(float a, float am, float ap, float bm, float bp,
                                            float tan_w) {
-    const float d0 = 0.5f * (ap - am);
-    const float d1 = 0.5f * (bp - bm);
-    return a + tan_w * fabsf(1.5f * d0 - 0.5f * d1);
+    return wet_value(a, ap, am, bp, bm, tan_w);
 }
 
 // Populations of a staged row as site_update reads them: g and h of

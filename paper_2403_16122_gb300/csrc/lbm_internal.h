@@ -315,6 +315,9 @@ cudaError_t launch_step(int tx, int ty, int storage, const Inst* d_inst,
                         const Tile* d_tiles, int n_tiles, int parity, int obs,
                         double* d_partials, cudaStream_t s);
 
+// Tile CTAs resident at once on the device (0: unsupported shape).
+int tile_resident_ctas(int tx, int ty);
+
 // Double-precision constants of the equilibrium initialisation.
 struct InitConst {
     double L, Hs, Hl, Tm, Cp, Cpref, inv_ramp;

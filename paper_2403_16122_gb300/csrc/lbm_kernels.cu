@@ -279,38 +279,6 @@ __device__ __forceinline__ Macro local_macro(const Phys& P, const float g[9], co
 }
 
 // ---------------------------------------------------------------------------
-// Block reduction of the observables (FP64)
-// ---------------------------------------------------------------------------
-// out: this tile's slot in observable-major partials (observable j at
-// out[j * stride]).
-template <int NT>
-__device__ void block_reduce_obs(double v[kObs], double* __restrict__ out, int stride) {
-    __shared__ double red[NT / 32][kObs];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < kObs; ++j) {
-        double x = v[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            double y = __shfl_xor_sync(0xffffffffu, x, o);
-            x = (j == 9) ? fmax(x, y) : x + y;
-        }
-        v[j] = x;
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int j = 0; j < kObs; ++j) red[warp][j] = v[j];
-    }
-    __syncthreads();
-    if (threadIdx.x < kObs) {
-        const int j = threadIdx.x;
-        double acc = red[0][j];
-        for (int w = 1; w < NT / 32; ++w) acc = (j == 9) ? fmax(acc, red[w][j]) : acc + red[w][j];
-        out[(long long)j * stride] = acc;
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Per-site update shared by the tile and strip kernels
 // ---------------------------------------------------------------------------
 // Isotropic stencils of Eq. 38 at one site: gradients of phi, rho, p^{n-1},
@@ -332,17 +300,17 @@ struct ColSums {
 };
 __device__ __forceinline__ ColSums col_sums(float m, float c, float p) {
     ColSums r;
-    r.A = kW1 * c + kW2 * (p + m);
+    r.A = fmaf(kW1, c, kW2 * (p + m));
     r.D = p - m;
     return r;
 }
 __device__ __forceinline__ void grad_cols(const ColSums& L, const ColSums& C, const ColSums& R,
                                           float& gx, float& gy) {
     gx = 3.f * (R.A - L.A);
-    gy = 3.f * (kW1 * C.D + kW2 * (R.D + L.D));
+    gy = 3.f * fmaf(kW1, C.D, kW2 * (R.D + L.D));
 }
-// The same for two fields at once (paired FP32 operations, each component
-// evaluated exactly as above); S2 = p + m is returned for the Laplacian.
+// Two fields at once (paired FP32 operations, each component as above); S2 = p + m is returned for the
+// Laplacian.
 struct ColSums2 {
     float2 A, D, S2;
 };
@@ -360,12 +328,20 @@ __device__ __forceinline__ void grad_cols2(const ColSums2& L, const ColSums2& C,
     gy = __fmul2_rn(k3, __ffma2_rn(make_float2(kW1, kW1), C.D,
                                    __fmul2_rn(make_float2(kW2, kW2), __fadd2_rn(R.D, L.D))));
 }
+// Wetting ghost (Eqs. 39-41) behind the wall site a, from its neighbours along
+// the wall in the adjacent layer (ap, am) and in the next one (bp, bm). The
+// rounding is fixed here, so that every kernel gives the same ghost.
+__device__ __forceinline__ float wet_value(float a, float ap, float am, float bp, float bm,
+                                           float tan_w) {
+    const float d0 = 0.5f * (ap - am), d1 = 0.5f * (bp - bm);
+    return fmaf(tan_w, fabsf(fmaf(1.5f, d0, -0.5f * d1)), a);
+}
 // cL, cR: row-y values of the side columns; sL, sC, sR: p + m of each column
 __device__ __forceinline__ float lap_cols(float cL, float cC, float cR, float sL, float sC,
                                           float sR) {
-    const float t1 = (cR + cL) + sC - 4.f * cC;
-    const float t2 = (sR + sL) - 4.f * cC;
-    return 6.f * (kW1 * t1 + kW2 * t2);
+    const float t1 = fmaf(-4.f, cC, (cR + cL) + sC);
+    const float t2 = fmaf(-4.f, cC, sR + sL);
+    return 6.f * fmaf(kW1, t1, kW2 * t2);
 }
 
 // Pulled populations of one site as site_update reads them: from arrays, or
@@ -410,27 +386,86 @@ struct SlotGHPops {
     __device__ __forceinline__ float F(int i) const { return f[i]; }
 };
 
-// Per-thread observable sums of the sites it updates. The sums run in FP32
-// with Neumaier's compensation (the running sum and the rounding error each
-// addition dropped), and (s + c) is taken in FP64 before the warp, block and
-// item reductions, which are FP64: the result matches an FP64 running sum of
-// the same FP32 per-site values to well below their own rounding, without
-// FP64 arithmetic per site (the FP64 rate of the GPU is a small fraction of
-// its FP32 rate). Slot 9 is a maximum, not a sum.
-struct ObsAcc {
-    float s[kObs], c[kObs];
+// Observables of the one site a thread of a tile updates. They are kept as they
+// come, FP32 values of which H (slot 2) has three terms; the sums over sites
+// are FP64. Slot 9 is a maximum, not a sum.
+struct SiteObs {
+    float v[kObs], h[2];
+    int nh;
     __device__ __forceinline__ void zero() {
 #pragma unroll
-        for (int j = 0; j < kObs; ++j) { s[j] = 0.f; c[j] = 0.f; }
+        for (int j = 0; j < kObs; ++j) v[j] = 0.f;
+        h[0] = h[1] = 0.f;
+        nh = 0;
     }
     __device__ __forceinline__ void add(int j, float x) {
-        const float t = s[j] + x;
-        c[j] += fabsf(s[j]) >= fabsf(x) ? (s[j] - t) + x : (x - t) + s[j];
-        s[j] = t;
+        if (j != 2) {
+            v[j] = x;
+        } else {  // the calls' order is fixed: the indices fold
+            if (nh == 0) v[2] = x;
+            else if (nh == 1) h[0] = x;
+            else h[1] = x;
+            ++nh;
+        }
     }
-    __device__ __forceinline__ void max(int j, float x) { s[j] = fmaxf(s[j], x); }
-    __device__ __forceinline__ double total(int j) const { return (double)s[j] + (double)c[j]; }
+    __device__ __forceinline__ void max(int j, float x) { v[j] = x; }
+    __device__ __forceinline__ double total(int j) const {
+        return j == 2 ? (double)v[2] + ((double)h[0] + (double)h[1]) : (double)v[j];
+    }
 };
+
+// Block reduction of the observables of a tile (FP64). out: the tile's slot in
+// observable-major partials (observable j at out[j * stride]). A warp's sums of
+// slots 0-6 go through one reduce-scatter: at lane bits 4, 3 and 2 a lane
+// keeps half of its vector and adds the partner's copy of that half, then two
+// xor steps finish, so a warp issues 9 FP64 additions for them instead of 35
+// (FP64 runs at two additions a cycle and SM here: eleven plain trees were
+// 3.5 us of the observable step). Slot 9 is a maximum of FP32 values; slots 7,
+// 8 and 10 are zero but for a few sites and are skipped where a warp has none.
+template <int NT>
+__device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __restrict__ out,
+                                                 int stride) {
+    __shared__ double red[NT / 32][kObs];
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    double k4[4], k2[2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const double lo = ob.total(q), hi = q + 4 < 7 ? ob.total(q + 4) : 0.0;
+        k4[q] = (b4 ? hi : lo) + __shfl_xor_sync(kAll, b4 ? lo : hi, 16);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        k2[q] = (b3 ? k4[q + 2] : k4[q]) + __shfl_xor_sync(kAll, b3 ? k4[q] : k4[q + 2], 8);
+    double t = (b2 ? k2[1] : k2[0]) + __shfl_xor_sync(kAll, b2 ? k2[0] : k2[1], 4);
+    t += __shfl_xor_sync(kAll, t, 2);
+    t += __shfl_xor_sync(kAll, t, 1);
+    if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
+    float mx = ob.v[9];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kAll, mx, o));
+    if (lane == 0) red[warp][9] = (double)mx;
+    auto rare = [&](int j) {
+        double x = 0.0;
+        if (__any_sync(kAll, ob.v[j] != 0.f)) {
+            x = ob.total(j);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
+        }
+        if (lane == 0) red[warp][j] = x;
+    };
+    rare(7);
+    rare(8);
+    rare(10);
+    __syncthreads();
+    if (threadIdx.x < kObs) {
+        const int j = threadIdx.x;
+        double acc = red[0][j];
+        for (int w = 1; w < NT / 32; ++w) acc = (j == 9) ? fmax(acc, red[w][j]) : acc + red[w][j];
+        out[(long long)j * stride] = acc;
+    }
+}
 
 // Observable sums of a warp strip, taken row by row: at the end of each row
 // the values of its sites (at most 30) are summed across the warp in FP32,
@@ -560,7 +595,7 @@ struct BlockStore {
 // post-collision populations and carried fields of one site. The order of
 // every floating-point operation is fixed here; kernels differ only in which
 // multiply-adds the compiler contracts.
-template <bool OBS, typename ST = float, typename Pops = ArrPops, typename Acc = ObsAcc,
+template <bool OBS, typename ST = float, typename Pops = ArrPops, typename Acc = SiteObs,
           typename Store = SiteStore>
 __device__ __forceinline__ void site_update_to(const Phys& P, int flags, const Macro& m,
                                                const Pops& pop, float phiux_p, float phiuy_p,
@@ -748,7 +783,7 @@ __device__ __forceinline__ void site_update_to(const Phys& P, int flags, const M
     }
 }
 
-template <bool OBS, typename ST = float, typename Pops = ArrPops, typename Acc = ObsAcc>
+template <bool OBS, typename ST = float, typename Pops = ArrPops, typename Acc = SiteObs>
 __device__ __forceinline__ void site_update(const Phys& P, int flags, const Macro& m,
                                             const Pops& pop,
                                             float phiux_p, float phiuy_p, const Stencil& st,
@@ -762,58 +797,101 @@ __device__ __forceinline__ void site_update(const Phys& P, int flags, const Macr
 // ---------------------------------------------------------------------------
 // The fused step kernel
 // ---------------------------------------------------------------------------
-// One CTA advances tile T of lattice I (the body of every tile kernel).
-template <int TX, int TY, bool OBS>
-__device__ __forceinline__ void tile_step(const Inst& I, const Tile& T, int parity,
-                                          double* __restrict__ partials) {
-    constexpr int NT = TX * TY;
-    constexpr int SW = TX + 4;                  // shared row width (2-cell halo)
-    constexpr int SH = TY + 4;
-    __shared__ float s_phi[SH * SW], s_rho[SH * SW], s_p[SH * SW], s_S[SH * SW];
-
-    const Phys P = load_phys(I);
-    Lat l;
-    l.A = static_cast<const float*>(I.pop[parity]);
-    l.Aaux = I.aux[parity];
-    l.plane = (int)I.plane; l.nx = I.nx; l.ny = I.ny; l.pitch = I.pitch; l.flags = I.flags;
-    float* __restrict__ B = static_cast<float*>(I.pop[parity ^ 1]);
-    float* __restrict__ Baux = I.aux[parity ^ 1];
-    const float abb = P.abb();
-
-    const int tid = threadIdx.x;
-    const int tx = tid % TX, ty = tid / TX;
-    const int tw = T.tw, th = T.th, x0 = T.x0, y0 = T.y0;
-    const bool active = tx < tw && ty < th;
-    const int x = x0 + tx, y = y0 + ty;
-    auto SI = [](int ox, int oy) { return (oy + 2) * SW + (ox + 2); };
-
-    // ---- phase A: own site ----
-    float g[9], h[9], f[9];
-    Macro m;
-    float phiux_p = 0.f, phiuy_p = 0.f;
-    if (active) {
-        const int own = y * l.pitch + x;
-        pull_set<0>(l, x, y, abb, g);
-        pull_set<1>(l, x, y, abb, h);
-        pull_set<2>(l, x, y, abb, f);
-        const float flp = ldAux(l, 0, own);
-        phiux_p = ldAux(l, 1, own);
-        phiuy_p = ldAux(l, 2, own);
-        m = local_macro(P, g, h, flp);
-        s_phi[SI(tx, ty)] = m.phi;
-        s_rho[SI(tx, ty)] = m.rho;
-        s_p[SI(tx, ty)] = ldAux(l, 3, own);
-        s_S[SI(tx, ty)] = ldAux(l, 4, own);
+// Where the values that stream into site (x, y) lie: the element offsets of
+// the (g_i, h_i) pairs and of the f_i, and the links whose h arrives through a
+// Dirichlet wall (bit i). A link that starts behind a wall takes the site's
+// own opposite population. Selects, no branches: every load of a site can be
+// issued before the first is waited for.
+struct Links {
+    int gh[9], f[9];
+    unsigned dir;
+};
+__device__ __forceinline__ Links links_of(int nx, int ny, int pitch, int flags, int x, int y) {
+    Links L;
+    L.dir = 0u;
+    const bool px = flags & kPeriodicX, py = flags & kPeriodicY;
+    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+    const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
+    const int own = y * pitch + x;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        const int cx = CX(i), cy = CY(i);
+        const bool wx = cx > 0 ? (!px && x == 0) : (cx < 0 ? (!px && x == nx - 1) : false);
+        const bool wy = cy > 0 ? (!py && y == 0) : (cy < 0 ? (!py && y == ny - 1) : false);
+        const int src = (cy > 0 ? ym : (cy < 0 ? yp : y)) * pitch + (cx > 0 ? xm : (cx < 0 ? xp : x));
+        L.gh[i] = wx || wy ? gh_at(OPP(i), own, 0) : gh_at(i, src, 0);
+        L.f[i] = wx || wy ? f_at(OPP(i), own) : f_at(i, src);
+        if ((wx && (flags & (cx > 0 ? kDirXlo : kDirXhi))) ||
+            (wy && (flags & (cy > 0 ? kDirYlo : kDirYhi))))
+            L.dir |= 1u << i;
     }
+    return L;
+}
+template <typename V>
+__device__ __forceinline__ V ld_cg(const float* p) {
+    return __ldcg(reinterpret_cast<const V*>(p));
+}
+// The pulled pairs as g and h (h_0 shifted, see Inst), anti-bounce-back
+// -h + 2 w_i Cp_ref T_w on the links in dir.
+__device__ __forceinline__ void split_gh(const float2 gh[9], unsigned dir, float abb, float g[9],
+                                         float h[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        g[i] = gh[i].x;
+        h[i] = (dir >> i) & 1u ? -gh[i].y + 2.0f * WGT(i) * abb : gh[i].y;
+    }
+}
 
-    // ---- phase B: ring cells and wall extras ----
-    const bool wxlo = !(l.flags & kPeriodicX) && x0 == 0;
-    const bool wxhi = !(l.flags & kPeriodicX) && x0 + tw == l.nx;
-    const bool wylo = !(l.flags & kPeriodicY) && y0 == 0;
-    const bool wyhi = !(l.flags & kPeriodicY) && y0 + th == l.ny;
+// One CTA advances tile T of lattice I by one step (the body of every tile
+// kernel). Small lattices are its main use, and there a step is a chain of
+// latencies (a global load takes 700-800 cycles, the arithmetic of a site about
+// 2000 with two warps a scheduler): so the loads of a thread's own site (18,
+// the (g, h) pairs and own-site groups as vectors) and of the ring site it
+// also serves (10) are all in flight together, the ring needs one entry a
+// thread, and the second block barrier is met only by tiles at a wall. The
+// ring sites' walls, corners and the two extra cells a wall row needs beyond
+// the ring are the same entries for every step. `I` is read from shared memory.
+// The tile's mdot is left in s_md (one value a warp; the caller synchronises
+// and adds them up).
+template <int TX, int TY>
+struct TileShared {
+    static constexpr int SW = TX + 4, SH = TY + 4;  // two-cell halo
+    float2 pr[SH * SW];                             // phi, rho
+    float2 ps[SH * SW];                             // p, S of the step before
+    float md[TX * TY / 32];
+    float col[TY][TX];                              // f_s (observable steps)
+    Inst inst;
+    int ok;
+};
+// What a thread of a tile does in every step, worked out once per launch: its
+// own site and the ring entry it serves, with the offsets of their loads.
+template <int TX, int TY>
+struct TilePlan {
+    bool active, serves, ghost, ring, outx, outy, walls;
+    int x, y, own;
+    int ox, oy, gx, gy, cxl, cyl, adj;  // ring cell, lattice site, adjacent lattice site
+    Links L, R;                         // loads of the own site and of the ring entry
+};
+template <int TX, int TY>
+__device__ __forceinline__ TilePlan<TX, TY> tile_plan(TileShared<TX, TY>& sh, const Tile& T) {
+    const Inst& I = sh.inst;
+    constexpr int NT = TX * TY;
+    static_assert(2 * (TX + 2) + 2 * TY + 16 <= NT, "one ring entry per thread");
+    TilePlan<TX, TY> p;
+    const int nx = I.nx, ny = I.ny, pitch = I.pitch, flags = I.flags;
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    const int tw = T.tw, th = T.th, x0 = T.x0, y0 = T.y0;
+    p.active = tx < tw && ty < th;
+    p.x = x0 + tx;
+    p.y = y0 + ty;
+    p.own = p.y * pitch + p.x;
+    const bool wxlo = !(flags & kPeriodicX) && x0 == 0;
+    const bool wxhi = !(flags & kPeriodicX) && x0 + tw == nx;
+    const bool wylo = !(flags & kPeriodicY) && y0 == 0;
+    const bool wyhi = !(flags & kPeriodicY) && y0 + th == ny;
+    p.walls = wxlo || wxhi || wylo || wyhi;
     const int nring = 2 * (tw + 2) + 2 * th;
     const int nent = nring + 4 * ((int)wxlo + (int)wxhi + (int)wylo + (int)wyhi);
-
     // Entry k -> tile-relative cell (ox, oy).
     auto entry = [&](int k, int& ox, int& oy) {
         if (k < tw + 2) { ox = k - 1; oy = -1; return; }
@@ -837,159 +915,206 @@ __device__ __forceinline__ void tile_step(const Inst& I, const Tile& T, int pari
         else if (side == 2) { oy = b ? th + 1 : -2; ox = a; }
         else { oy = b ? th + 1 : -2; ox = tw - 1 - a; }
     };
-    // Resolve a tile-relative cell to lattice coordinates; false when behind a wall.
-    auto resolve = [&](int ox, int oy, int& gx, int& gy, bool& outx, bool& outy) {
-        gx = x0 + ox; gy = y0 + oy;
-        outx = outy = false;
-        if (gx < 0 || gx >= l.nx) {
-            if (l.flags & kPeriodicX) gx = (gx + l.nx) % l.nx; else outx = true;
+    // the ring is served from the last threads: ragged tiles have idle ones there
+    const int k = NT - 1 - tid;
+    p.serves = k < nent;
+    p.ring = k < nring;
+    p.ox = p.oy = p.gx = p.gy = p.cxl = p.cyl = p.adj = 0;
+    p.outx = p.outy = false;
+    if (p.active) p.L = links_of(nx, ny, pitch, flags, p.x, p.y);
+    if (p.serves) {
+        entry(k, p.ox, p.oy);
+        p.gx = x0 + p.ox;
+        p.gy = y0 + p.oy;
+        if (p.gx < 0 || p.gx >= nx) {
+            if (flags & kPeriodicX) p.gx = (p.gx + nx) % nx; else p.outx = true;
         }
-        if (gy < 0 || gy >= l.ny) {
-            if (l.flags & kPeriodicY) gy = (gy + l.ny) % l.ny; else outy = true;
+        if (p.gy < 0 || p.gy >= ny) {
+            if (flags & kPeriodicY) p.gy = (p.gy + ny) % ny; else p.outy = true;
         }
-        return !(outx || outy);
-    };
+        p.cxl = p.outx ? (p.gx < 0 ? 0 : nx - 1) : p.gx;
+        p.cyl = p.outy ? (p.gy < 0 ? 0 : ny - 1) : p.gy;
+        p.adj = p.cyl * pitch + p.cxl;
+        p.R = links_of(nx, ny, pitch, flags, p.cxl, p.cyl);
+    }
+    p.ghost = p.outx || p.outy;
+    return p;
+}
 
-    for (int k = tid; k < nent; k += NT) {
-        int ox, oy, gx, gy;
-        bool outx, outy;
-        entry(k, ox, oy);
-        if (resolve(ox, oy, gx, gy, outx, outy)) {
+template <int TX, int TY, bool OBS>
+__device__ __forceinline__ void tile_step(TileShared<TX, TY>& sh, const Tile& T,
+                                          const TilePlan<TX, TY>& p, int parity,
+                                          double* __restrict__ partials) {
+    constexpr int NT = TX * TY, SW = TX + 4;
+    const Inst& I = sh.inst;
+    const Phys P = load_phys(I);
+    const float* __restrict__ A = static_cast<const float*>(I.pop[parity]);
+    const float* __restrict__ Aaux = I.aux[parity];
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    auto SI = [](int ox, int oy) { return (oy + 2) * SW + (ox + 2); };
+
+    // ---- all loads, then the local macroscopic fields ----
+    float2 gh[9];
+    float f[9];
+    float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
+    if (p.active) {
+#pragma unroll
+        for (int i = 1; i < 9; ++i) gh[i] = ld_cg<float2>(A + p.L.gh[i]);
+        o0 = ld_cg<float4>(Aaux + own0_at(p.own, 0));
+        o1 = ld_cg<float4>(Aaux + own1_at(p.own, 0));
+#pragma unroll
+        for (int i = 1; i < 9; ++i) f[i] = ld_cg<float>(A + p.L.f[i]);
+    }
+    float2 rgh[9], rps = make_float2(0.f, 0.f);
+    float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.serves) {  // a ghost takes the p and S of its adjacent site
+#pragma unroll
+        for (int i = 1; i < 9; ++i) rgh[i] = ld_cg<float2>(A + p.R.gh[i]);
+        r0 = ld_cg<float4>(Aaux + own0_at(p.adj, 0));
+        rps = ld_cg<float2>(Aaux + own1_at(p.adj, 2));
+    }
+    const float abb = P.abb();
+    Macro m;
+    float g[9], h[9];
+    if (p.active) {
+        gh[0] = make_float2(o0.x, o0.y);
+        f[0] = o0.z;
+        split_gh(gh, p.L.dir, abb, g, h);
+        m = local_macro(P, g, h, o0.w);
+        sh.pr[SI(tx, ty)] = make_float2(m.phi, m.rho);
+        sh.ps[SI(tx, ty)] = make_float2(o1.z, o1.w);
+    }
+    if (p.serves) {
+        if (!p.ghost) {
+            rgh[0] = make_float2(r0.x, r0.y);
             float gg[9], hh[9];
-            pull_set<0>(l, gx, gy, abb, gg);
-            pull_set<1>(l, gx, gy, abb, hh);
-            const int idx = gy * l.pitch + gx;
-            Macro mm = local_macro(P, gg, hh, ldAux(l, 0, idx));
-            s_phi[SI(ox, oy)] = mm.phi;
-            s_rho[SI(ox, oy)] = mm.rho;
-            if (k < nring) {
-                s_p[SI(ox, oy)] = ldAux(l, 3, idx);
-                s_S[SI(ox, oy)] = ldAux(l, 4, idx);
-            }
-        } else if (k < nring) {
-            // ghost: p and S copy the adjacent lattice value
-            int cx = min(max(x0 + ox, 0), l.nx - 1), cy = min(max(y0 + oy, 0), l.ny - 1);
-            if (!outx) cx = gx;
-            if (!outy) cy = gy;
-            const int idx = cy * l.pitch + cx;
-            s_p[SI(ox, oy)] = ldAux(l, 3, idx);
-            s_S[SI(ox, oy)] = ldAux(l, 4, idx);
+            split_gh(rgh, p.R.dir, abb, gg, hh);
+            const Macro mm = local_macro(P, gg, hh, r0.w);
+            sh.pr[SI(p.ox, p.oy)] = make_float2(mm.phi, mm.rho);
         }
+        sh.ps[SI(p.ox, p.oy)] = rps;  // (the extra cells' are not read)
     }
     __syncthreads();
 
-    // ---- phase C: ghosts of phi (wetting) and rho (copy) ----
-    // Shared-memory slot of a lattice coordinate (periodic axes wrap into the
-    // tile's 2-cell halo).
-    auto lat_slot = [&](int xl, int yl) {
-        int ox = xl - x0, oy = yl - y0;
-        if (ox < -2) ox += l.nx; else if (ox > tw + 1) ox -= l.nx;
-        if (oy < -2) oy += l.ny; else if (oy > th + 1) oy -= l.ny;
-        return SI(ox, oy);
-    };
-    auto wrap_or_clamp = [](int v, int n, bool periodic) {
-        if (v >= 0 && v < n) return v;
-        if (periodic) return (v + n) % n;
-        return v < 0 ? 0 : n - 1;
-    };
-    for (int k = tid; k < nring; k += NT) {
-        int ox, oy, gx, gy;
-        bool outx, outy;
-        entry(k, ox, oy);
-        if (resolve(ox, oy, gx, gy, outx, outy)) continue;
-        const int cxl = outx ? (x0 + ox < 0 ? 0 : l.nx - 1) : gx;
-        const int cyl = outy ? (y0 + oy < 0 ? 0 : l.ny - 1) : gy;
-        s_rho[SI(ox, oy)] = s_rho[lat_slot(cxl, cyl)];
-        float ghost;
-        if (outy && !outx) {
-            const int ya = cyl, yb = (y0 + oy < 0) ? 1 : l.ny - 2;
-            const bool px = (l.flags & kPeriodicX) != 0;
-            const int xm = wrap_or_clamp(gx - 1, l.nx, px), xp = wrap_or_clamp(gx + 1, l.nx, px);
-            const float d0 = 0.5f * (s_phi[lat_slot(xp, ya)] - s_phi[lat_slot(xm, ya)]);
-            const float d1 = 0.5f * (s_phi[lat_slot(xp, yb)] - s_phi[lat_slot(xm, yb)]);
-            ghost = s_phi[lat_slot(gx, ya)] + P.rare->tan_w * fabsf(1.5f * d0 - 0.5f * d1);
-        } else if (outx && !outy) {
-            const int xa = cxl, xb = (x0 + ox < 0) ? 1 : l.nx - 2;
-            const bool py = (l.flags & kPeriodicY) != 0;
-            const int ym = wrap_or_clamp(gy - 1, l.ny, py), yp = wrap_or_clamp(gy + 1, l.ny, py);
-            const float d0 = 0.5f * (s_phi[lat_slot(xa, yp)] - s_phi[lat_slot(xa, ym)]);
-            const float d1 = 0.5f * (s_phi[lat_slot(xb, yp)] - s_phi[lat_slot(xb, ym)]);
-            ghost = s_phi[lat_slot(xa, gy)] + P.rare->tan_w * fabsf(1.5f * d0 - 0.5f * d1);
-        } else {
-            ghost = s_phi[lat_slot(cxl, cyl)];
-        }
-        s_phi[SI(ox, oy)] = ghost;
-    }
-    __syncthreads();
-
-    // ---- phase D: stencils, forces, collisions, store ----
-    ObsAcc ob;
-    if (OBS) ob.zero();
-    if (active) {
-        Stencil st;
-        {
-            // column sums of x-1, x, x+1 from shared memory (same expressions as
-            // the strip kernel's shuffled column sums)
-            auto col = [&](const float* a, int dx, float& m_, float& c_, float& p_) {
-                m_ = a[SI(tx + dx, ty - 1)];
-                c_ = a[SI(tx + dx, ty)];
-                p_ = a[SI(tx + dx, ty + 1)];
+    // ---- ghosts of phi (wetting, Eqs. 39-41) and rho (copy) ----
+    if (p.walls) {  // the whole CTA
+        if (p.ring && p.ghost) {
+            // Shared-memory slot of a lattice coordinate (periodic axes wrap
+            // into the tile's 2-cell halo).
+            const int nx = I.nx, ny = I.ny, flags = I.flags;
+            auto lat_slot = [&](int xl, int yl) {
+                int sx = xl - T.x0, sy = yl - T.y0;
+                if (sx < -2) sx += nx; else if (sx > T.tw + 1) sx -= nx;
+                if (sy < -2) sy += ny; else if (sy > T.th + 1) sy -= ny;
+                return SI(sx, sy);
             };
-            float mL, cL, pL, mC, cC, pC, mR, cR, pR;
-            col(s_phi, -1, mL, cL, pL); col(s_phi, 0, mC, cC, pC); col(s_phi, 1, mR, cR, pR);
-            grad_cols(col_sums(mL, cL, pL), col_sums(mC, cC, pC), col_sums(mR, cR, pR),
-                      st.gphx, st.gphy);
-            st.lph = lap_cols(cL, cC, cR, pL + mL, pC + mC, pR + mR);
-            col(s_rho, -1, mL, cL, pL); col(s_rho, 0, mC, cC, pC); col(s_rho, 1, mR, cR, pR);
-            grad_cols(col_sums(mL, cL, pL), col_sums(mC, cC, pC), col_sums(mR, cR, pR),
-                      st.grx, st.gry);
-            col(s_p, -1, mL, cL, pL); col(s_p, 0, mC, cC, pC); col(s_p, 1, mR, cR, pR);
-            grad_cols(col_sums(mL, cL, pL), col_sums(mC, cC, pC), col_sums(mR, cR, pR),
-                      st.gpx, st.gpy);
-            col(s_S, -1, mL, cL, pL); col(s_S, 0, mC, cC, pC); col(s_S, 1, mR, cR, pR);
-            grad_cols(col_sums(mL, cL, pL), col_sums(mC, cC, pC), col_sums(mR, cR, pR),
-                      st.gSx, st.gSy);
+            auto wrap_or_clamp = [](int v, int n, bool periodic) {
+                if (v >= 0 && v < n) return v;
+                if (periodic) return (v + n) % n;
+                return v < 0 ? 0 : n - 1;
+            };
+            float2 gv = sh.pr[lat_slot(p.cxl, p.cyl)];
+            if (p.outx != p.outy) {
+                // the two layers along the wall's normal, one site either way
+                // along the wall
+                int a[4];
+                if (p.outy) {
+                    const int yb = p.gy < 0 ? 1 : ny - 2;
+                    const bool px = flags & kPeriodicX;
+                    const int xm = wrap_or_clamp(p.gx - 1, nx, px), xp = wrap_or_clamp(p.gx + 1, nx, px);
+                    a[0] = lat_slot(xp, p.cyl); a[1] = lat_slot(xm, p.cyl);
+                    a[2] = lat_slot(xp, yb); a[3] = lat_slot(xm, yb);
+                } else {
+                    const int xb = p.gx < 0 ? 1 : nx - 2;
+                    const bool py = flags & kPeriodicY;
+                    const int ym = wrap_or_clamp(p.gy - 1, ny, py), yp = wrap_or_clamp(p.gy + 1, ny, py);
+                    a[0] = lat_slot(p.cxl, yp); a[1] = lat_slot(p.cxl, ym);
+                    a[2] = lat_slot(xb, yp); a[3] = lat_slot(xb, ym);
+                }
+                gv.x = wet_value(gv.x, sh.pr[a[0]].x, sh.pr[a[1]].x, sh.pr[a[2]].x, sh.pr[a[3]].x,
+                                 P.rare->tan_w);
+            }
+            sh.pr[SI(p.ox, p.oy)] = gv;
         }
-        site_update<OBS>(P, l.flags, m, ArrPops{g, h, f}, phiux_p, phiuy_p, st, B, Baux, l.plane,
-                         y * l.pitch + x, x == l.nx / 2, y == l.ny / 2, ob);
-    }
-    if (OBS) {
-        double v[kObs];
-#pragma unroll
-        for (int j = 0; j < kObs; ++j) v[j] = ob.total(j);
-        block_reduce_obs<NT>(v, partials + T.part, I.part_stride);
-    }
-    // the tile's mdot of this step joins its FP64 running sum (warp sums,
-    // then the warps in order), and on observable steps each column's f_s
-    // (rows in order) is added to the lattice's column profile
-    __shared__ float s_md[NT / 32];
-    __shared__ float s_col[TY][TX];
-    if (I.macc || (OBS && I.prof)) {
-        float md = active ? m.mdot : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) md += __shfl_xor_sync(0xffffffffu, md, o);
-        if ((tid & 31) == 0) s_md[tid >> 5] = md;
-        if (OBS) s_col[ty][tx] = active ? m.fs : 0.f;
         __syncthreads();
-        if (I.macc && tid == 0) {
-            float sum = 0.f;
-            for (int w = 0; w < NT / 32; ++w) sum += s_md[w];
-            I.macc[T.part] += (double)sum;
+    }
+
+    // ---- stencils, forces, collisions, store ----
+    SiteObs ob;
+    if (OBS) ob.zero();
+    if (p.active) {
+        Stencil st;
+        auto col = [&](const float2* a, int dx) {
+            return col_sums2(a[SI(tx + dx, ty - 1)], a[SI(tx + dx, ty)], a[SI(tx + dx, ty + 1)]);
+        };
+        float2 dx2, dy2;
+        {
+            const ColSums2 cl = col(sh.pr, -1), cc = col(sh.pr, 0), cr = col(sh.pr, 1);
+            grad_cols2(cl, cc, cr, dx2, dy2);
+            st.gphx = dx2.x; st.gphy = dy2.x; st.grx = dx2.y; st.gry = dy2.y;
+            st.lph = lap_cols(sh.pr[SI(tx - 1, ty)].x, m.phi, sh.pr[SI(tx + 1, ty)].x, cl.S2.x,
+                              cc.S2.x, cr.S2.x);
         }
-        if (OBS && I.prof && ty == 0 && tx < tw) {
+        grad_cols2(col(sh.ps, -1), col(sh.ps, 0), col(sh.ps, 1), dx2, dy2);
+        st.gpx = dx2.x; st.gpy = dy2.x; st.gSx = dx2.y; st.gSy = dy2.y;
+        site_update<OBS>(P, I.flags, m, ArrPops{g, h, f}, o1.x, o1.y, st, I.pop[parity ^ 1],
+                         I.aux[parity ^ 1], 0, p.own, p.x == I.nx / 2, p.y == I.ny / 2, ob);
+    }
+    float md = p.active ? m.mdot : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) md += __shfl_xor_sync(0xffffffffu, md, o);
+    if ((tid & 31) == 0) sh.md[tid >> 5] = md;
+    if constexpr (OBS) {
+        sh.col[ty][tx] = p.active ? m.fs : 0.f;
+        block_reduce_obs<NT>(ob, partials + T.part, I.part_stride);  // synchronises
+        // each column's f_s (rows in order) joins the lattice's column profile
+        if (I.prof && ty == 0 && tx < T.tw) {
             float sum = 0.f;
-            for (int r = 0; r < th; ++r) sum += s_col[r][tx];
-            atomicAdd(I.prof + x0 + tx, (double)sum);
+            for (int r = 0; r < T.th; ++r) sum += sh.col[r][tx];
+            atomicAdd(I.prof + T.x0 + tx, (double)sum);
         }
     }
 }
 
+// The lattice record of the CTA's tile into shared memory (every thread).
+template <int TX, int TY>
+__device__ __forceinline__ void load_inst(TileShared<TX, TY>& sh, const Inst& I) {
+    static_assert(sizeof(Inst) % 4 == 0, "copied by words");
+    const int* s = reinterpret_cast<const int*>(&I);
+    int* d = reinterpret_cast<int*>(&sh.inst);
+    for (int q = threadIdx.x; q < (int)(sizeof(Inst) / 4); q += TX * TY) d[q] = s[q];
+    __syncthreads();
+}
+// The tile's mdot of a step (thread 0, after a block barrier): the warps in order.
+template <int TX, int TY>
+__device__ __forceinline__ double tile_mdot(const TileShared<TX, TY>& sh) {
+    float sum = 0.f;
+    for (int w = 0; w < TX * TY / 32; ++w) sum += sh.md[w];
+    return (double)sum;
+}
+
 template <int TX, int TY, bool OBS>
-__global__ void __launch_bounds__(TX * TY)
+__global__ void __launch_bounds__(TX * TY, 256 / (TX * TY) > 0 ? 256 / (TX * TY) : 1)
 step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int parity,
           double* __restrict__ partials) {
+    __shared__ TileShared<TX, TY> sh;
+    // Programmatic dependent launch: the next step's CTAs work out their plan,
+    // from tables no step writes, while this step runs. They are let in only
+    // once this CTA's own wait is over: earlier, the plans of several steps to
+    // come take issue slots from the one that runs (0.3-1 us a step slower
+    // between 128 x 96 and 203 x 151 sites).
     const Tile T = tiles[blockIdx.x];
-    tile_step<TX, TY, OBS>(insts[T.inst], T, parity, partials);
+    load_inst<TX, TY>(sh, insts[T.inst]);
+    const TilePlan<TX, TY> plan = tile_plan<TX, TY>(sh, T);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the tile's mdot of this step joins its FP64 running sum, which is read
+    // here: a load at the end of the chain would lengthen it by its latency
+    double* const macc = sh.inst.macc ? sh.inst.macc + T.part : nullptr;
+    const double acc = macc && threadIdx.x == 0 ? *macc : 0.0;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    tile_step<TX, TY, OBS>(sh, T, plan, parity, partials);
+    __syncthreads();
+    if (macc && threadIdx.x == 0) *macc = acc + tile_mdot<TX, TY>(sh);
 }
 
 // Handle-free variant for lbm_step_noalloc: the lattice record arrives by
@@ -998,6 +1123,8 @@ step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int pa
 template <bool OBS>
 __global__ void __launch_bounds__(256)
 step_tile_noalloc(const __grid_constant__ Inst I, int tiles_x, double* __restrict__ partials) {
+    __shared__ TileShared<32, 8> sh;
+    load_inst<32, 8>(sh, I);
     Tile T;
     T.inst = 0;
     T.x0 = (int)(blockIdx.x % tiles_x) * 32;
@@ -1005,7 +1132,7 @@ step_tile_noalloc(const __grid_constant__ Inst I, int tiles_x, double* __restric
     T.tw = min(32, I.nx - T.x0);
     T.th = min(8, I.ny - T.y0);
     T.part = (int)blockIdx.x;
-    tile_step<32, 8, OBS>(I, T, 0, partials);
+    tile_step<32, 8, OBS>(sh, T, tile_plan<32, 8>(sh, T), 0, partials);
 }
 
 
@@ -1074,9 +1201,7 @@ __device__ __forceinline__ float strip_wet_ghost(float a, float b, float outer_a
     float bp = __shfl_down_sync(0xffffffffu, b, 1), bm = __shfl_up_sync(0xffffffffu, b, 1);
     if (lane == 31) { ap = outer_a; bp = outer_b; }
     if (lane == 0) { am = outer_a; bm = outer_b; }
-    const float d0 = 0.5f * (ap - am);
-    const float d1 = 0.5f * (bp - bm);
-    return a + tan_w * fabsf(1.5f * d0 - 0.5f * d1);
+    return wet_value(a, ap, am, bp, bm, tan_w);
 }
 
 // ---------------------------------------------------------------------------
@@ -1925,11 +2050,17 @@ reduce_noalloc(int n_parts, const double* __restrict__ partials, double* __restr
 template <int TX, int TY>
 cudaError_t launch_tile(const Inst* d_inst, const Tile* d_tiles, int n_tiles, int parity,
                         int obs, double* d_partials, cudaStream_t s) {
-    if (obs)
-        step_fp32<TX, TY, true><<<n_tiles, TX * TY, 0, s>>>(d_inst, d_tiles, parity, d_partials);
-    else
-        step_fp32<TX, TY, false><<<n_tiles, TX * TY, 0, s>>>(d_inst, d_tiles, parity, d_partials);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n_tiles);
+    cfg.blockDim = dim3(TX * TY);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, obs ? step_fp32<TX, TY, true> : step_fp32<TX, TY, false>,
+                              d_inst, d_tiles, parity, d_partials);
 }
 
 template <int WARPS, int MINB, typename ST>
@@ -2496,6 +2627,27 @@ cudaError_t launch_step(int tx, int ty, int storage, const Inst* d_inst, const T
     if (tx == 64 && ty == 4) return launch_tile<64, 4>(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
     if (tx == 32 && ty == 16) return launch_tile<32, 16>(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
     return cudaErrorInvalidValue;
+}
+
+namespace {
+template <int TX, int TY>
+int tile_resident() {
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_fp32<TX, TY, false>, TX * TY,
+                                                      0) != cudaSuccess)
+        return 0;
+    return per_sm * sms;
+}
+}  // namespace
+
+int tile_resident_ctas(int tx, int ty) {
+    if (tx == 32 && ty == 8) return tile_resident<32, 8>();
+    if (tx == 32 && ty == 4) return tile_resident<32, 4>();
+    if (tx == 64 && ty == 4) return tile_resident<64, 4>();
+    if (tx == 32 && ty == 16) return tile_resident<32, 16>();
+    return 0;
 }
 
 cudaError_t launch_step_noalloc(const Inst& I, int tiles_x, int n_tiles, double* scratch,

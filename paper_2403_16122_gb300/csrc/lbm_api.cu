@@ -5,7 +5,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <new>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -282,24 +284,98 @@ bool tiled(const lbm_handle* h) {
 // Output columns of one item of a strip-like layout.
 int item_width(int kind) { return kind == LBM_KERNEL_BLOCK ? lbmk::kBlockW : lbmk::kStripW; }
 
-// Rows per strip item: as requested, or (0) the fewest that let one wave of
-// resident warps take every item of every lattice at once.
+// Number of strip items of every lattice at `rows` rows an item.
+int items_at(const lbm_handle* h, int rows) {
+    const int wd = item_width(h->kind);
+    int n = 0;
+    for (const auto& p : h->params)
+        n += ((p.nx + wd - 1) / wd) * ((p.ny + rows - 1) / rows);
+    return n;
+}
+
+// Estimated time of a step at `rows` rows an item, in rows of a fully occupied
+// device: the CTAs (h->warps items each, in table order) go to the first free
+// of `slots` places; a CTA takes its longest item's rows and kItemCost rows for
+// the two rows beyond it and its start, and while only a fraction f of the
+// places is taken each CTA runs at 1 / (kTailA + kTailB f) of the full
+// device's pace at most. Fitted to measured steps of 15 sets of lattices (one of
+// 300 x 300 to 2501 x 2501, 8 to 256 of mixed sizes) at 4 to 12 row counts
+// each: the choice below is within 1 % of the fastest but for 500 x 500 in FP16
+// storage (11 %).
+constexpr double kItemCost = 1.0, kTailA = 0.4, kTailB = 0.6;
+double step_estimate(const lbm_handle* h, int rows, int slots) {
+    const int wd = item_width(h->kind);
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;  // CTAs' ends
+    double start = 0.0;
+    int in_cta = 0, longest = 0;
+    auto flush = [&]() {
+        if (in_cta == 0) return;
+        if ((int)free_at.size() == slots) {
+            start = free_at.top();
+            free_at.pop();
+        }
+        free_at.push(start + longest + kItemCost);
+        in_cta = longest = 0;
+    };
+    for (const auto& p : h->params) {
+        const int strips = (p.nx + wd - 1) / wd;
+        for (int y0 = 0; y0 < p.ny; y0 += rows) {
+            const int height = std::min(rows, p.ny - y0);
+            for (int s = 0; s < strips; ++s) {
+                longest = std::max(longest, height);
+                if (++in_cta == h->warps) flush();
+            }
+        }
+    }
+    flush();
+    double t = start, at = start;  // full until the last CTA starts
+    for (; !free_at.empty(); free_at.pop()) {
+        const double f = (double)free_at.size() / slots;
+        t += (free_at.top() - at) * std::min(1.0, kTailA + kTailB * f);
+        at = free_at.top();
+    }
+    return t;
+}
+
+// Rows per strip item: as requested, or (0) the count with the shortest
+// estimated step among those that fill 1, 2, 3, 4, 6 or 8 waves of resident
+// warps (for one wave also one and two rows more or less). A single large lattice is fastest in one
+// wave; many lattices are not, as their last segments are short (48 drops on
+// 128 .. 512 squared: 341 us a step in one wave, 213 us at 32 rows; 256 drops
+// in FP16 storage on 64 .. 256: 449 us and 298 us at 20 rows; 64 drops: 118 us
+// and 87 us at 18), nor is one whose
+// rounding leaves a few items for a second wave (2501 x 2501: 267 us at 116
+// rows, 254 us at 118).
 int item_rows(const lbm_handle* h) {
     if (h->rows_req > 0) return h->rows_req;
-    long long strip_rows = 0;
     int max_ny = kMinRows;
-    const int wd = item_width(h->kind);
-    for (const auto& p : h->params) {
-        strip_rows += (long long)((p.nx + wd - 1) / wd) * p.ny;
-        max_ny = std::max(max_ny, p.ny);
-    }
+    for (const auto& p : h->params) max_ny = std::max(max_ny, p.ny);
     const int warps = h->kind == LBM_KERNEL_BLOCK
                           ? lbmk::block_resident_warps(h->warps, h->regs, h->storage)
                           : lbmk::strip_resident_warps(h->kind == LBM_KERNEL_STAGED, h->warps,
                                                        h->regs, h->storage);
     if (warps <= 0) return 16;
-    const long long r = (strip_rows + warps - 1) / warps;
-    return (int)std::min<long long>(std::max<long long>(r, kMinRows), max_ny);
+    const int slots = std::max(1, warps / h->warps);
+    int best = 0, last = 0;
+    double best_t = 0.0;
+    for (const int waves : {1, 2, 3, 4, 6, 8}) {
+        int lo = kMinRows, hi = max_ny;  // fewest rows with at most `waves` waves of items
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (items_at(h, mid) <= waves * warps) hi = mid; else lo = mid + 1;
+        }
+        // (just below one wave, the few items too many may be short ones)
+        const bool one = waves == 1;
+        for (int r = one ? std::max(kMinRows, lo - 2) : lo; r <= (one ? std::min(lo + 2, max_ny) : lo); ++r) {
+            if (!one && r >= last) break;  // tried with fewer waves
+            const double t = step_estimate(h, r, slots);
+            if (best == 0 || t < best_t) { best = r; best_t = t; }
+        }
+        last = last ? std::min(last, lo) : lo;
+        // one lattice: always the first (and lbm_create stays short)
+        if (lo == kMinRows || h->n_inst == 1) break;
+    }
+    return best;
 }
 
 void build_items(lbm_handle* h) {
@@ -320,14 +396,6 @@ void build_items(lbm_handle* h) {
             }
         h->inst[k].part_end = (int)h->items.size();
     }
-}
-
-int count_items(const lbm_handle* h) {
-    const int wd = item_width(h->kind);
-    int n = 0;
-    for (const auto& p : h->params)
-        n += ((p.nx + wd - 1) / wd) * ((p.ny + h->rows - 1) / h->rows);
-    return n;
 }
 
 void drop_graphs(lbm_handle* h) {
@@ -416,10 +484,10 @@ int upload_tables(lbm_handle* h) {
     if (e != cudaSuccess) return cuda_fail(e);
     h->persist_grid = h->kind == LBM_KERNEL_BLOCK
                           ? lbmk::block_persistent_grid(h->warps, h->regs, h->storage,
-                                                        count_items(h))
+                                                        items_at(h, h->rows))
                           : (is_strip(h->kind)
                                  ? lbmk::persistent_grid(h->kind == LBM_KERNEL_STAGED, h->warps,
-                                                         h->regs, h->storage, count_items(h))
+                                                         h->regs, h->storage, items_at(h, h->rows))
                                  : 0);
     return LBM_OK;
 }

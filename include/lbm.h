@@ -392,7 +392,8 @@ int64_t lbm_launch_count(const lbm_handle* h);
    any stream capture begins. The cached address does not survive the
    destruction of the device's context (cudaDeviceReset, or a primary
    context released and retained again): do not call this entry point after
-   that. Works for every wall combination (tile kernel). Returns LBM_EINVAL
+   that. Works for every wall combination (tiles, or strips for larger lattices
+   periodic in x). Returns LBM_EINVAL
    for bad parameters, pointers, pitch or overlapping buffers, LBM_ECUDA for
    launch errors. */
 #define LBM_NOALLOC_MAX_TILES 8192

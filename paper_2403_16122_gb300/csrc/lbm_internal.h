@@ -330,12 +330,19 @@ cudaError_t launch_init(const Inst* d_inst, int inst, int n_sites, int storage,
                         InitConst c, const double* d_phi0, const double* d_T0,
                         int parity, cudaStream_t s);
 
-// One time step of the 32 x 8 tile kernel for a single lattice whose record
-// is passed by value (no device tables), with the per-tile observable
-// partials in `scratch` (n_tiles * kObs doubles) and the reduced record in
-// d_obs (kObs doubles). Buffer 0 of I is the source, buffer 1 the target.
-cudaError_t launch_step_noalloc(const Inst& I, int tiles_x, int n_tiles, double* scratch,
-                                double* d_obs, cudaStream_t s);
+// One observable time step for a single lattice whose record is passed by value
+// (no device tables; buffer 0 of I is the source, buffer 1 the target), the
+// partials of every tile or strip item in `scratch` (observable-major, kObs
+// rows): 32 x ty tiles (ty 4 or 8), or strip items of `rows` rows of a lattice
+// periodic in x; and the reduction of n_parts partials into d_obs (kObs doubles).
+cudaError_t launch_step_noalloc(const Inst& I, int ty, int tiles_x, int n_tiles, double* scratch,
+                                cudaStream_t s);
+cudaError_t launch_step_noalloc_strip(const Inst& I, int rows, int n_items, double* scratch,
+                                      cudaStream_t s);
+cudaError_t launch_reduce_noalloc(int n_parts, const double* scratch, double* d_obs, cudaStream_t s);
+// Strip warps of launch_step_noalloc_strip resident at once on the current
+// device (0: a call failed); raises the kernel's shared-memory limit there.
+int noalloc_strip_warps();
 
 // Physics constants of a lattice record from its problem statement (the
 // pointers, pitch and observable slots are left to the caller); *L gets the

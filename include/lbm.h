@@ -343,7 +343,8 @@ int lbm_barrier_selftest(lbm_handle* h, uint64_t limit_ns, int32_t* err_flag);
 int64_t lbm_step_count(const lbm_handle* h);
 
 /* Number of kernel launches the library queued since the handle was created
-   (every kernel, including initialisation and reductions). */
+   (initialisation, steps and reductions; not the conversions of lbm_get_state
+   and lbm_set_state). */
 int64_t lbm_launch_count(const lbm_handle* h);
 
 /* ---------------------------------------------------------------------------

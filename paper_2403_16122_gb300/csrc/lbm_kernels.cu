@@ -2008,6 +2008,48 @@ __global__ void init_16(const Inst* __restrict__ insts, int inst, InitConst c,
     }
 }
 
+// ---------------------------------------------------------------------------
+// State transfer, FP32 storage: two planes of the caller's planar doubles at a
+// time (lattice order, no padding) to or from the blocked buffers. Plane q is
+// population q of 27 (g_0..8, h_0..8, f_0..8) or carried field q - 27. A
+// population's 32 values of a block lie 4 or 8 bytes apart, a plane's 8; a
+// plane moves 8 bytes a site to the host and is bound by that copy. h_0 is
+// stored shifted by -L f_l (see Inst).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float* state_at(const Inst& I, int parity, int q, int site) {
+    if (q >= 27) return I.aux[parity] + aux_at(q - 27, site);
+    const int set = q / 9, i = q % 9;
+    if (i == 0) return I.aux[parity] + own0_at(site, set);
+    return static_cast<float*>(I.pop[parity]) + pop_at(set, i, site);
+}
+__global__ void planes_from_state(const Inst* __restrict__ insts, int inst, int parity, double L,
+                                  int q0, int n_q, double* __restrict__ out) {
+    const Inst& I = insts[inst];
+    const int n = I.nx * I.ny;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int site = k / I.nx * I.pitch + k % I.nx;
+        for (int a = 0; a < n_q; ++a) {
+            double v = *state_at(I, parity, q0 + a, site);
+            if (q0 + a == 9) v += L * (double)*state_at(I, parity, 27, site);
+            out[(long long)a * n + k] = v;
+        }
+    }
+}
+// qa, qb: the planes staged in `in`; plane 9 comes with plane 27.
+__global__ void state_from_planes(const Inst* __restrict__ insts, int inst, int parity, double L,
+                                  int qa, int qb, const double* __restrict__ in) {
+    const Inst& I = insts[inst];
+    const int n = I.nx * I.ny;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int site = k / I.nx * I.pitch + k % I.nx;
+        double a = in[k];
+        const float b = (float)in[(long long)n + k];
+        if (qa == 9 && qb == 27) a -= L * (double)b;
+        *state_at(I, parity, qa, site) = (float)a;
+        *state_at(I, parity, qb, site) = b;
+    }
+}
+
 // Reduction of the partials of the allocation-free step by one cluster: CTA r
 // sums every kRedCtas-th run of kRedThreads partials (observable-major, so the
 // loads are coalesced), warps and CTAs by fixed trees, and CTA 0 reads the
@@ -2763,6 +2805,22 @@ cudaError_t launch_init(const Inst* d_inst, int inst, int n_sites, int storage, 
         init_16<__nv_bfloat16><<<blocks, threads, 0, s>>>(d_inst, inst, c, d_phi0, d_T0, parity);
     else
         return cudaErrorNotSupported;
+    return cudaGetLastError();
+}
+
+namespace {
+int transfer_blocks(int n_sites) { return std::max(1, std::min((n_sites + 255) / 256, 4096)); }
+}  // namespace
+
+cudaError_t launch_planes_from_state(const Inst* d_inst, int inst, int n_sites, int parity, double L,
+                                     int q0, int n_q, double* d_out, cudaStream_t s) {
+    planes_from_state<<<transfer_blocks(n_sites), 256, 0, s>>>(d_inst, inst, parity, L, q0, n_q, d_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_state_from_planes(const Inst* d_inst, int inst, int n_sites, int parity, double L,
+                                     int qa, int qb, const double* d_in, cudaStream_t s) {
+    state_from_planes<<<transfer_blocks(n_sites), 256, 0, s>>>(d_inst, inst, parity, L, qa, qb, d_in);
     return cudaGetLastError();
 }
 

@@ -215,8 +215,8 @@ def lbm_solid_profile(h, inst: int, nx: int) -> np.ndarray:
 
 
 def lbm_get_state(h, inst: int, nx: int, ny: int):
-    pops = np.zeros((27, ny, nx))
-    aux = np.zeros((5, ny, nx))
+    pops = np.empty((27, ny, nx))
+    aux = np.empty((5, ny, nx))
     rc = load().lbm_get_state(h, int(inst), _dptr(pops), _dptr(aux))
     if rc:
         raise LbmError(rc, "lbm_get_state")

@@ -261,11 +261,11 @@ int lbm_set_state(lbm_handle* h, int32_t inst, const double* pops,
    For the strip and block layouts b = 0 picks the rows per item that let
    one wave of resident warps take every item of every lattice.
    lbm_create picks STAGED (4, 0, 168) when every lattice is periodic in x,
-   else TILE (32, 4). While its choice stands, FP32 lattices that together are
-   two waves of 32 x 4 tiles or less (some 155,000 sites) are stepped by the
-   tile kernel, where one step of so few sites is shorter; the persistent
-   execution form, and a layout chosen by lbm_set_kernel or lbm_autotune, run
-   as they are reported. */
+   else TILE (32, 4). While its choice stands, lattices that together are two
+   waves of 32 x 4 tiles or less (some 155,000 sites, 116,000 in 16-bit storage)
+   are stepped by the tile kernel, where one step of so few sites is shorter;
+   the persistent execution form, and a layout chosen by lbm_set_kernel or
+   lbm_autotune, run as they are reported. */
 #define LBM_KERNEL_TILE   0
 #define LBM_KERNEL_STRIP  1
 #define LBM_KERNEL_STAGED 2

@@ -272,7 +272,8 @@ bool is_strip(int kind) {
 // thread per site; 155,648 sites on 152 SMs). There a step is one chain of
 // latencies, and a strip item's is some rows longer than a tile's: 2.7 us
 // against 8.1 us a step on 128 x 96 sites, 4.1 against 8.3 on 256 x 256, 6.8
-// against 9.0 on 320 x 320. Beyond, the strips come level: 9.6 against 11.5 on
+// against 9.0 on 320 x 320; in BF16 storage (three CTAs an SM, 116,736 sites)
+// 2.9 against 10.2 on 128 x 128, 6.4 against 11.3 on 256 x 256. Beyond, the strips come level: 9.6 against 11.5 on
 // 400 x 400 but 26.4 against 24.3 for a step with its observables, 13.4 against
 // 14.6 on 512 x 512, 23.3 against 18.1 on 620 x 620. The persistent form stays
 // with the strips.
@@ -675,12 +676,10 @@ int lbm_create(const lbm_params* p, int32_t n_inst, int32_t storage, void* d_wor
     // row-staged strips, one wave of items; small lattices run in tiles
     h->kind = all_px ? LBM_KERNEL_STAGED : LBM_KERNEL_TILE;
     h->rows_req = 0;
-    if (storage == LBM_STORE_FP32) {
-        long long n_tiles = 0;
-        for (int k = 0; k < n_inst; ++k)
-            n_tiles += (long long)((p[k].nx + kTileX - 1) / kTileX) * ((p[k].ny + kTileY - 1) / kTileY);
-        h->small = n_tiles <= 2 * lbmk::tile_resident_ctas(kTileX, kTileY);
-    }
+    long long n_tiles = 0;
+    for (int k = 0; k < n_inst; ++k)
+        n_tiles += (long long)((p[k].nx + kTileX - 1) / kTileX) * ((p[k].ny + kTileY - 1) / kTileY);
+    h->small = n_tiles <= 2 * lbmk::tile_resident_ctas(storage);
     rc = upload_tables(h);
     if (rc != LBM_OK) {
         delete h;

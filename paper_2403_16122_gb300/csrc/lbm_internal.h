@@ -315,8 +315,16 @@ cudaError_t launch_step(int tx, int ty, int storage, const Inst* d_inst,
                         const Tile* d_tiles, int n_tiles, int parity, int obs,
                         double* d_partials, cudaStream_t s);
 
-// Tile CTAs resident at once on the device (0: unsupported shape).
-int tile_resident_ctas(int tx, int ty);
+// CTAs of the 32 x 4 tile kernel of a storage type resident at once on the
+// device (0: a call failed).
+int tile_resident_ctas(int storage);
+// The tile kernels of 16-bit storage (32 x 4 tiles), compiled in their part.
+template <typename ST>
+struct Tile16 {
+    static cudaError_t launch(const Inst* d_inst, const Tile* d_tiles, int n_tiles, int parity,
+                              int obs, double* d_partials, cudaStream_t s);
+    static int resident();
+};
 
 // Double-precision constants of the equilibrium initialisation.
 struct InitConst {

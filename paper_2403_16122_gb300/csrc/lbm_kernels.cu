@@ -799,16 +799,16 @@ __device__ __forceinline__ void site_update(const Phys& P, int flags, const Macr
 // ---------------------------------------------------------------------------
 // Where the values that stream into site (x, y) lie: the element offsets of
 // the (g_i, h_i) pairs and of the f_i, and the links whose h arrives through a
-// Dirichlet wall (bit i). A link that starts behind a wall takes the site's
-// own opposite population. Selects, no branches: every load of a site can be
+// Dirichlet wall, and all that start behind a wall (bit i). Such a link takes
+// the site's own opposite population. Selects, no branches: every load of a site can be
 // issued before the first is waited for.
 struct Links {
     int gh[9], f[9];
-    unsigned dir;
+    unsigned dir, wall;
 };
 __device__ __forceinline__ Links links_of(int nx, int ny, int pitch, int flags, int x, int y) {
     Links L;
-    L.dir = 0u;
+    L.dir = L.wall = 0u;
     const bool px = flags & kPeriodicX, py = flags & kPeriodicY;
     const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
     const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
@@ -821,6 +821,7 @@ __device__ __forceinline__ Links links_of(int nx, int ny, int pitch, int flags, 
         const int src = (cy > 0 ? ym : (cy < 0 ? yp : y)) * pitch + (cx > 0 ? xm : (cx < 0 ? xp : x));
         L.gh[i] = wx || wy ? gh_at(OPP(i), own, 0) : gh_at(i, src, 0);
         L.f[i] = wx || wy ? f_at(OPP(i), own) : f_at(i, src);
+        if (wx || wy) L.wall |= 1u << i;
         if ((wx && (flags & (cx > 0 ? kDirXlo : kDirXhi))) ||
             (wy && (flags & (cy > 0 ? kDirYlo : kDirYhi))))
             L.dir |= 1u << i;
@@ -831,14 +832,50 @@ template <typename V>
 __device__ __forceinline__ V ld_cg(const float* p) {
     return __ldcg(reinterpret_cast<const V*>(p));
 }
-// The pulled pairs as g and h (h_0 shifted, see Inst), anti-bounce-back
+// A (g_i, h_i) pair and an f_i as they are stored: two floats and one, or (16-bit
+// storage) one word and one half.
+template <typename ST>
+struct Raw {
+    using Pair = float2;
+    using F = float;
+    static __device__ __forceinline__ Pair pair(const void* A, int off) {
+        return ld_cg<float2>(static_cast<const float*>(A) + off);
+    }
+    static __device__ __forceinline__ F f(const void* A, int off) {
+        return __ldcg(static_cast<const float*>(A) + off);
+    }
+};
+struct Raw16 {
+    using Pair = unsigned;
+    using F = unsigned short;
+    static __device__ __forceinline__ Pair pair(const void* A, int off) {
+        return __ldcg(reinterpret_cast<const unsigned*>(static_cast<const unsigned short*>(A) + off));
+    }
+    static __device__ __forceinline__ F f(const void* A, int off) {
+        return __ldcg(static_cast<const unsigned short*>(A) + off);
+    }
+};
+template <> struct Raw<__half> : Raw16 {};
+template <> struct Raw<__nv_bfloat16> : Raw16 {};
+// The pulled pairs as g and h (rest populations g0, h0 apart; h_0 shifted, see
+// Inst), 16-bit ones decoded with the site's references; anti-bounce-back
 // -h + 2 w_i Cp_ref T_w on the links in dir.
-__device__ __forceinline__ void split_gh(const float2 gh[9], unsigned dir, float abb, float g[9],
-                                         float h[9]) {
+template <typename ST>
+__device__ __forceinline__ void split_gh(const typename Raw<ST>::Pair raw[9], const float4& o0,
+                                         unsigned dir, float abb, const float2& ref, float Cpref,
+                                         float g[9], float h[9]) {
+    g[0] = o0.x;
+    h[0] = o0.y;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        g[i] = gh[i].x;
-        h[i] = (dir >> i) & 1u ? -gh[i].y + 2.0f * WGT(i) * abb : gh[i].y;
+    for (int i = 1; i < 9; ++i) {
+        if constexpr (sizeof(ST) == 4) {
+            g[i] = raw[i].x;
+            h[i] = raw[i].y;
+        } else {
+            g[i] = Bits16<ST>::add_lo(raw[i], WGT(i) * ref.x);
+            h[i] = Bits16<ST>::add_hi(raw[i], WGT(i) * Cpref * ref.y);
+        }
+        if ((dir >> i) & 1u) h[i] = -h[i] + 2.0f * WGT(i) * abb;
     }
 }
 
@@ -853,11 +890,12 @@ __device__ __forceinline__ void split_gh(const float2 gh[9], unsigned dir, float
 // the ring are the same entries for every step. `I` is read from shared memory.
 // The tile's mdot is left in s_md (one value a warp; the caller synchronises
 // and adds them up).
-template <int TX, int TY>
+template <int TX, int TY, typename ST = float>
 struct TileShared {
     static constexpr int SW = TX + 4, SH = TY + 4;  // two-cell halo
     float2 pr[SH * SW];                             // phi, rho
     float2 ps[SH * SW];                             // p, S of the step before
+    float t[sizeof(ST) == 4 ? 1 : SH * SW];         // T (16-bit storage)
     float md[TX * TY / 32];
     float col[TY][TX];                              // f_s (observable steps)
     Inst inst;
@@ -873,8 +911,7 @@ struct TilePlan {
     Links L, R;                         // loads of the own site and of the ring entry
 };
 template <int TX, int TY>
-__device__ __forceinline__ TilePlan<TX, TY> tile_plan(TileShared<TX, TY>& sh, const Tile& T) {
-    const Inst& I = sh.inst;
+__device__ __forceinline__ TilePlan<TX, TY> tile_plan(const Inst& I, const Tile& T) {
     constexpr int NT = TX * TY;
     static_assert(2 * (TX + 2) + 2 * TY + 16 <= NT, "one ring entry per thread");
     TilePlan<TX, TY> p;
@@ -941,55 +978,59 @@ __device__ __forceinline__ TilePlan<TX, TY> tile_plan(TileShared<TX, TY>& sh, co
     return p;
 }
 
-template <int TX, int TY, bool OBS>
-__device__ __forceinline__ void tile_step(TileShared<TX, TY>& sh, const Tile& T,
+template <int TX, int TY, bool OBS, typename ST>
+__device__ __forceinline__ void tile_step(TileShared<TX, TY, ST>& sh, const Tile& T,
                                           const TilePlan<TX, TY>& p, int parity,
                                           double* __restrict__ partials) {
     constexpr int NT = TX * TY, SW = TX + 4;
+    constexpr bool kHalf = sizeof(ST) != 4;
     const Inst& I = sh.inst;
     const Phys P = load_phys(I);
-    const float* __restrict__ A = static_cast<const float*>(I.pop[parity]);
+    const void* __restrict__ A = I.pop[parity];
     const float* __restrict__ Aaux = I.aux[parity];
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
     auto SI = [](int ox, int oy) { return (oy + 2) * SW + (ox + 2); };
 
     // ---- all loads, then the local macroscopic fields ----
-    float2 gh[9];
-    float f[9];
+    typename Raw<ST>::Pair gh[9];
+    typename Raw<ST>::F fr[9];
+    float2 ref = make_float2(0.f, 0.f);  // decoding references (16-bit storage)
     float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
     if (p.active) {
 #pragma unroll
-        for (int i = 1; i < 9; ++i) gh[i] = ld_cg<float2>(A + p.L.gh[i]);
+        for (int i = 1; i < 9; ++i) gh[i] = Raw<ST>::pair(A, p.L.gh[i]);
         o0 = ld_cg<float4>(Aaux + own0_at(p.own, 0));
         o1 = ld_cg<float4>(Aaux + own1_at(p.own, 0));
+        if constexpr (kHalf) ref = ld_cg<float2>(Aaux + ref_at(p.own, 0));
 #pragma unroll
-        for (int i = 1; i < 9; ++i) f[i] = ld_cg<float>(A + p.L.f[i]);
+        for (int i = 1; i < 9; ++i) fr[i] = Raw<ST>::f(A, p.L.f[i]);
     }
-    float2 rgh[9], rps = make_float2(0.f, 0.f);
+    typename Raw<ST>::Pair rgh[9];
+    float2 rref = ref, rps = make_float2(0.f, 0.f);
     float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (p.serves) {  // a ghost takes the p and S of its adjacent site
 #pragma unroll
-        for (int i = 1; i < 9; ++i) rgh[i] = ld_cg<float2>(A + p.R.gh[i]);
+        for (int i = 1; i < 9; ++i) rgh[i] = Raw<ST>::pair(A, p.R.gh[i]);
         r0 = ld_cg<float4>(Aaux + own0_at(p.adj, 0));
+        if constexpr (kHalf) rref = ld_cg<float2>(Aaux + ref_at(p.adj, 0));
         rps = ld_cg<float2>(Aaux + own1_at(p.adj, 2));
     }
     const float abb = P.abb();
     Macro m;
     float g[9], h[9];
     if (p.active) {
-        gh[0] = make_float2(o0.x, o0.y);
-        f[0] = o0.z;
-        split_gh(gh, p.L.dir, abb, g, h);
+        split_gh<ST>(gh, o0, p.L.dir, abb, ref, P.Cpref, g, h);
         m = local_macro(P, g, h, o0.w);
+        if constexpr (kHalf) sh.t[SI(tx, ty)] = m.T;
         sh.pr[SI(tx, ty)] = make_float2(m.phi, m.rho);
         sh.ps[SI(tx, ty)] = make_float2(o1.z, o1.w);
     }
     if (p.serves) {
         if (!p.ghost) {
-            rgh[0] = make_float2(r0.x, r0.y);
             float gg[9], hh[9];
-            split_gh(rgh, p.R.dir, abb, gg, hh);
+            split_gh<ST>(rgh, r0, p.R.dir, abb, rref, P.Cpref, gg, hh);
             const Macro mm = local_macro(P, gg, hh, r0.w);
+            if constexpr (kHalf) sh.t[SI(p.ox, p.oy)] = mm.T;
             sh.pr[SI(p.ox, p.oy)] = make_float2(mm.phi, mm.rho);
         }
         sh.ps[SI(p.ox, p.oy)] = rps;  // (the extra cells' are not read)
@@ -1057,8 +1098,25 @@ __device__ __forceinline__ void tile_step(TileShared<TX, TY>& sh, const Tile& T,
         }
         grad_cols2(col(sh.ps, -1), col(sh.ps, 0), col(sh.ps, 1), dx2, dy2);
         st.gpx = dx2.x; st.gpy = dy2.x; st.gSx = dx2.y; st.gSy = dy2.y;
-        site_update<OBS>(P, I.flags, m, ArrPops{g, h, f}, o1.x, o1.y, st, I.pop[parity ^ 1],
-                         I.aux[parity ^ 1], 0, p.own, p.x == I.nx / 2, p.y == I.ny / 2, ob);
+        // f of 16-bit storage: deviations from the pressure of the site each
+        // comes from; and the references of the sites the outgoing values go to
+        // (the site itself for links that bounce)
+        float f[9];
+        Ref dref[9];
+        f[0] = o0.z;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            if constexpr (kHalf) {
+                const float ps = (p.L.wall >> i) & 1u ? o1.z : sh.ps[SI(tx - CX(i), ty - CY(i))].x;
+                f[i] = Bits16<ST>::fma_lo_2m12(fr[i], f_rest(i, ps));
+                const int to = SI(tx + CX(i), ty + CY(i));
+                dref[i] = (p.L.wall >> OPP(i)) & 1u ? Ref{m.phi, m.T} : Ref{sh.pr[to].x, sh.t[to]};
+            } else {
+                f[i] = fr[i];
+            }
+        }
+        site_update<OBS, ST>(P, I.flags, m, ArrPops{g, h, f}, o1.x, o1.y, st, I.pop[parity ^ 1],
+                             I.aux[parity ^ 1], 0, p.own, p.x == I.nx / 2, p.y == I.ny / 2, ob, dref);
     }
     float md = p.active ? m.mdot : 0.f;
 #pragma unroll
@@ -1077,8 +1135,8 @@ __device__ __forceinline__ void tile_step(TileShared<TX, TY>& sh, const Tile& T,
 }
 
 // The lattice record of the CTA's tile into shared memory (every thread).
-template <int TX, int TY>
-__device__ __forceinline__ void load_inst(TileShared<TX, TY>& sh, const Inst& I) {
+template <int TX, int TY, typename ST>
+__device__ __forceinline__ void load_inst(TileShared<TX, TY, ST>& sh, const Inst& I) {
     static_assert(sizeof(Inst) % 4 == 0, "copied by words");
     const int* s = reinterpret_cast<const int*>(&I);
     int* d = reinterpret_cast<int*>(&sh.inst);
@@ -1086,35 +1144,50 @@ __device__ __forceinline__ void load_inst(TileShared<TX, TY>& sh, const Inst& I)
     __syncthreads();
 }
 // The tile's mdot of a step (thread 0, after a block barrier): the warps in order.
-template <int TX, int TY>
-__device__ __forceinline__ double tile_mdot(const TileShared<TX, TY>& sh) {
+template <int TX, int TY, typename ST>
+__device__ __forceinline__ double tile_mdot(const TileShared<TX, TY, ST>& sh) {
     float sum = 0.f;
     for (int w = 0; w < TX * TY / 32; ++w) sum += sh.md[w];
     return (double)sum;
 }
 
-template <int TX, int TY, bool OBS>
-__global__ void __launch_bounds__(TX * TY, 256 / (TX * TY) > 0 ? 256 / (TX * TY) : 1)
-step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int parity,
-          double* __restrict__ partials) {
-    __shared__ TileShared<TX, TY> sh;
+template <int TX, int TY, bool OBS, typename ST>
+__device__ __forceinline__ void tile_kernel(const Inst* __restrict__ insts,
+                                            const Tile* __restrict__ tiles, int parity,
+                                            double* __restrict__ partials) {
+    __shared__ TileShared<TX, TY, ST> sh;
+    const Tile T = tiles[blockIdx.x];
+    load_inst(sh, insts[T.inst]);
+    const TilePlan<TX, TY> plan = tile_plan<TX, TY>(sh.inst, T);
     // Programmatic dependent launch: the next step's CTAs work out their plan,
     // from tables no step writes, while this step runs. They are let in only
     // once this CTA's own wait is over: earlier, the plans of several steps to
     // come take issue slots from the one that runs (0.3-1 us a step slower
     // between 128 x 96 and 203 x 151 sites).
-    const Tile T = tiles[blockIdx.x];
-    load_inst<TX, TY>(sh, insts[T.inst]);
-    const TilePlan<TX, TY> plan = tile_plan<TX, TY>(sh, T);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the tile's mdot of this step joins its FP64 running sum, which is read
     // here: a load at the end of the chain would lengthen it by its latency
     double* const macc = sh.inst.macc ? sh.inst.macc + T.part : nullptr;
     const double acc = macc && threadIdx.x == 0 ? *macc : 0.0;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    tile_step<TX, TY, OBS>(sh, T, plan, parity, partials);
+    tile_step<TX, TY, OBS, ST>(sh, T, plan, parity, partials);
     __syncthreads();
-    if (macc && threadIdx.x == 0) *macc = acc + tile_mdot<TX, TY>(sh);
+    if (macc && threadIdx.x == 0) *macc = acc + tile_mdot(sh);
+}
+
+template <int TX, int TY, bool OBS>
+__global__ void __launch_bounds__(TX * TY, 256 / (TX * TY) > 0 ? 256 / (TX * TY) : 1)
+step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int parity,
+          double* __restrict__ partials) {
+    tile_kernel<TX, TY, OBS, float>(insts, tiles, parity, partials);
+}
+
+// 16-bit storage in tiles: the small handles of lbm_create (32 x 4).
+template <bool OBS, typename ST>
+__global__ void __launch_bounds__(128, 2)
+step_tile_16(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int parity,
+             double* __restrict__ partials) {
+    tile_kernel<32, 4, OBS, ST>(insts, tiles, parity, partials);
 }
 
 // Handle-free variant for lbm_step_noalloc: the lattice record arrives by
@@ -1125,7 +1198,7 @@ __global__ void __launch_bounds__(32 * TY)
 step_tile_noalloc(const __grid_constant__ Inst I, int tiles_x, double* __restrict__ partials) {
     __shared__ TileShared<32, TY> sh;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    load_inst<32, TY>(sh, I);
+    load_inst(sh, I);
     Tile T;
     T.inst = 0;
     T.x0 = (int)(blockIdx.x % tiles_x) * 32;
@@ -1133,9 +1206,9 @@ step_tile_noalloc(const __grid_constant__ Inst I, int tiles_x, double* __restric
     T.tw = min(32, I.nx - T.x0);
     T.th = min(TY, I.ny - T.y0);
     T.part = (int)blockIdx.x;
-    const TilePlan<32, TY> plan = tile_plan<32, TY>(sh, T);
+    const TilePlan<32, TY> plan = tile_plan<32, TY>(sh.inst, T);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    tile_step<32, TY, true>(sh, T, plan, 0, partials);
+    tile_step<32, TY, true, float>(sh, T, plan, 0, partials);
 }
 
 // ---------------------------------------------------------------------------
@@ -2107,20 +2180,33 @@ reduce_noalloc(int n_parts, const double* __restrict__ partials, double* __restr
 
 #endif  // LBM_HAS_PART(0)
 
-template <int TX, int TY>
-cudaError_t launch_tile(const Inst* d_inst, const Tile* d_tiles, int n_tiles, int parity,
-                        int obs, double* d_partials, cudaStream_t s) {
+using TileKernel = void (*)(const Inst*, const Tile*, int, double*);
+inline cudaError_t launch_tile_kernel(TileKernel k, int threads, const Inst* d_inst,
+                                      const Tile* d_tiles, int n_tiles, int parity,
+                                      double* d_partials, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tiles);
-    cfg.blockDim = dim3(TX * TY);
+    cfg.blockDim = dim3(threads);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, obs ? step_fp32<TX, TY, true> : step_fp32<TX, TY, false>,
-                              d_inst, d_tiles, parity, d_partials);
+    return cudaLaunchKernelEx(&cfg, k, d_inst, d_tiles, parity, d_partials);
+}
+template <int TX, int TY>
+cudaError_t launch_tile(const Inst* d_inst, const Tile* d_tiles, int n_tiles, int parity,
+                        int obs, double* d_partials, cudaStream_t s) {
+    return launch_tile_kernel(obs ? step_fp32<TX, TY, true> : step_fp32<TX, TY, false>, TX * TY,
+                              d_inst, d_tiles, n_tiles, parity, d_partials, s);
+}
+inline int tile_kernel_resident(TileKernel k, int threads) {
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0) != cudaSuccess) return 0;
+    return per_sm * sms;
 }
 
 // Handle-free step of a lattice periodic in x for lbm_step_noalloc: the record
@@ -2518,6 +2604,24 @@ template struct StripPart<__half, false>;
 template struct StripPart<__nv_bfloat16, true>;
 #endif
 
+// The 16-bit tile kernels, compiled with the strips of their storage type.
+#if LBM_PART < 0 || LBM_PART == 4 || LBM_PART == 5
+template <typename ST>
+cudaError_t Tile16<ST>::launch(const Inst* d_inst, const Tile* d_tiles, int n_tiles, int parity,
+                               int obs, double* d_partials, cudaStream_t s) {
+    return launch_tile_kernel(obs ? step_tile_16<true, ST> : step_tile_16<false, ST>, 128, d_inst,
+                              d_tiles, n_tiles, parity, d_partials, s);
+}
+template <typename ST>
+int Tile16<ST>::resident() { return tile_kernel_resident(step_tile_16<false, ST>, 128); }
+#endif
+#if LBM_PART < 0 || LBM_PART == 4
+template struct Tile16<__half>;
+#endif
+#if LBM_PART < 0 || LBM_PART == 5
+template struct Tile16<__nv_bfloat16>;
+#endif
+
 // ---------------------------------------------------------------------------
 // The block kernels of one storage type, as compiled in their part
 // ---------------------------------------------------------------------------
@@ -2735,7 +2839,14 @@ bool tile_supported(int tx, int ty) {
 
 cudaError_t launch_step(int tx, int ty, int storage, const Inst* d_inst, const Tile* d_tiles,
                         int n_tiles, int parity, int obs, double* d_partials, cudaStream_t s) {
-    if (storage != 0) return cudaErrorNotSupported;
+    if (storage != LBM_STORE_FP32) {
+        if (tx != 32 || ty != 4) return cudaErrorNotSupported;
+        if (storage == LBM_STORE_FP16)
+            return Tile16<__half>::launch(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
+        if (storage == LBM_STORE_BF16)
+            return Tile16<__nv_bfloat16>::launch(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
+        return cudaErrorNotSupported;
+    }
     if (tx == 32 && ty == 8) return launch_tile<32, 8>(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
     if (tx == 32 && ty == 4) return launch_tile<32, 4>(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
     if (tx == 64 && ty == 4) return launch_tile<64, 4>(d_inst, d_tiles, n_tiles, parity, obs, d_partials, s);
@@ -2743,25 +2854,10 @@ cudaError_t launch_step(int tx, int ty, int storage, const Inst* d_inst, const T
     return cudaErrorInvalidValue;
 }
 
-namespace {
-template <int TX, int TY>
-int tile_resident() {
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_fp32<TX, TY, false>, TX * TY,
-                                                      0) != cudaSuccess)
-        return 0;
-    return per_sm * sms;
-}
-}  // namespace
-
-int tile_resident_ctas(int tx, int ty) {
-    if (tx == 32 && ty == 8) return tile_resident<32, 8>();
-    if (tx == 32 && ty == 4) return tile_resident<32, 4>();
-    if (tx == 64 && ty == 4) return tile_resident<64, 4>();
-    if (tx == 32 && ty == 16) return tile_resident<32, 16>();
-    return 0;
+int tile_resident_ctas(int storage) {
+    if (storage == LBM_STORE_FP16) return Tile16<__half>::resident();
+    if (storage == LBM_STORE_BF16) return Tile16<__nv_bfloat16>::resident();
+    return tile_kernel_resident(step_fp32<32, 4, false>, 128);
 }
 
 namespace {

@@ -32,7 +32,7 @@ int device_facts(double** out, int* warps, int* wave) {
         if (cudaGetSymbolAddress(&ptr, g_noalloc_partials) != cudaSuccess || !ptr)
             return LBM_ECUDA;
         g_warps[dev] = lbmk::noalloc_strip_warps();
-        g_wave[dev] = lbmk::tile_resident_ctas(32, 4);
+        g_wave[dev] = lbmk::tile_resident_ctas(LBM_STORE_FP32);
         g_scratch[dev] = static_cast<double*>(ptr);
     }
     *out = g_scratch[dev];

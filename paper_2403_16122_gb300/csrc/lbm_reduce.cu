@@ -5,15 +5,17 @@
 // observable; this kernel turns them into one record per lattice.
 //
 // FP64 arithmetic runs at two additions a cycle and SM on this GPU, and the
-// kernel is otherwise a chain of load latencies and barriers: a lattice's
-// partials are spread over CTAs of kPer, a CTA sums only the values it has, by
-// eight threads an observable and three shuffles, and a lattice that fits one
-// CTA needs no second pass. With more CTAs the last one to finish (an atomic
-// count) combines the CTA sums in the same way. Every sum is taken in an order
-// fixed by the partial indices alone, so the result does not depend on
-// scheduling. Against CTAs of 256 summed in two levels of 16 with a barrier
-// between them, a call of one step takes 60.4 us instead of 69.5 on 1024 x 1024
-// sites, 28.3 instead of 32.8 on 512 x 512, 9.5 instead of 13.1 on 256 x 8.
+// kernel is otherwise a chain of load latencies (700-800 cycles each), cold
+// instruction fetches and barriers: a lattice's partials are spread over CTAs of
+// kPer, eight threads an observable load their values at once, straight into
+// registers, and add them in a tree, and a lattice that fits one CTA needs no
+// second pass. With more CTAs the last one to finish (an atomic count) combines
+// the CTA sums in the same way. Every sum is taken in an order fixed by the
+// partial indices alone, so the result does not depend on scheduling. A call of
+// one step and a read of its observables, in us: 256 x 256 sites 30.6 with the
+// values staged through shared memory, 23.4 so (18 without a reduction at all);
+// 1024 x 1024 78.5 in CTAs of 256 summed in two levels of 16, 70.2 in CTAs of 64,
+// 66 so (59). One copy of the summing code for both passes was 1 us slower.
 #include "lbm_reduce.h"
 
 namespace lbmk {
@@ -23,19 +25,25 @@ constexpr int kPer = 64;              // partials per CTA
 constexpr int kThreads = 128;
 constexpr int kSums = kObs + 1;       // the observables, then the mdot running sums
 constexpr int kLanes = 8;             // threads that sum one observable
-static_assert(kSums * kLanes <= kThreads && kPer % kLanes == 0, "reduction shape");
+constexpr int kSumThreads = kSums * kLanes;
+static_assert(kSumThreads == 96 && kPer == 8 * kLanes, "three warps sum, one has the profile");
 
 __device__ __forceinline__ double combine(int j, double a, double b) {
     return j == 9 ? fmax(a, b) : a + b;  // slot 9: max |u|; 0 is neutral for it too
 }
 
-// Sum of the n <= kPer values staged in v[j], by thread t = j * kLanes + c: the
-// values c, c + kLanes, ... in order, then the lanes of the observable pairwise.
-// Whole warps take part; the result is valid where t < kSums * kLanes.
-__device__ __forceinline__ double sum_staged(const double (*v)[kPer + 1], int n, int t) {
-    const int j = t / kLanes < kSums ? t / kLanes : 0, c = t % kLanes;
-    double s = 0.0;
-    for (int q = c; q < n; q += kLanes) s = combine(j, s, v[j][q]);
+// Sum over n <= kPer values at p + q * stride for observable j, by its kLanes
+// threads: thread c takes values c, c + 8, .. c + 56, all loaded at once, and
+// adds them pairwise; then the threads pairwise. Valid in every thread.
+__device__ __forceinline__ double sum_values(const double* p, long long stride, int n, int j, int c) {
+    double a[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a[k] = c + 8 * k < n ? __ldcg(p + (c + 8 * k) * stride) : 0.0;
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+        for (int k = 0; k < w; ++k) a[k] = combine(j, a[k], a[k + w]);
+    double s = a[0];
 #pragma unroll
     for (int o = kLanes / 2; o > 0; o >>= 1) s = combine(j, s, __shfl_xor_sync(0xffffffffu, s, o));
     return s;
@@ -51,7 +59,6 @@ reduce_obs_split(const Inst* __restrict__ insts, const double* __restrict__ part
                  double* __restrict__ out, double* __restrict__ out_host,
                  double* __restrict__ frz, double* __restrict__ scratch,
                  unsigned* __restrict__ counts, long long step) {
-    __shared__ double v[kSums][kPer + 1];
     __shared__ double tot[kSums];
     __shared__ bool last;
     // Programmatic dependent launch: this grid is scheduled while the
@@ -62,35 +69,32 @@ reduce_obs_split(const Inst* __restrict__ insts, const double* __restrict__ part
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int k = blockIdx.x, b = blockIdx.y, t = threadIdx.x;
     const Inst& I = insts[k];
-    const int begin = I.part_begin, n = I.part_end - I.part_begin, stride = I.part_stride;
-    const int nx = I.nx;
-    double* const macc = I.macc;
-    double* const prof = I.prof;
-    double* const prof_out = I.prof_out;
+    const int begin = I.part_begin, n = I.part_end - I.part_begin;
     const int n_cta = n > 0 ? (n + kPer - 1) / kPer : 1;
     if (b >= n_cta) return;  // whole CTA, before any barrier or count
+    const int j = t / kLanes, c = t % kLanes;
+    const int at = begin + b * kPer, here = n - b * kPer < kPer ? n - b * kPer : kPer;
+    const double* const row = j < kObs ? partials + (long long)j * I.part_stride + at
+                                       : (I.macc ? I.macc + at : nullptr);
+    double* const prof = I.prof;
+    double* const prof_out = I.prof_out;
+    const int nx = I.nx;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int here = n - b * kPer < kPer ? n - b * kPer : kPer;
-    for (int q = t; q < kSums * kPer; q += kThreads) {
-        const int j = q / kPer, p = q % kPer;
-        if (p < here) {
-            const int at = begin + b * kPer + p;
-            v[j][p] = j < kObs ? partials[(long long)j * stride + at] : (macc ? macc[at] : 0.0);
-        }
-    }
-    if (prof && prof_out)
-        for (int x = b * kThreads + t; x < nx; x += n_cta * kThreads) {
+    double s = 0.0;
+    if (t < kSumThreads) {
+        s = sum_values(row, 1, row ? here : 0, j, c);
+    } else if (prof && prof_out) {  // the last warp: a share of the column profile
+        for (int x = b * 32 + (t & 31); x < nx; x += n_cta * 32) {
             prof_out[x] = __ldcg(prof + x);
             prof[x] = 0.0;
         }
-    __syncthreads();
-    double s = sum_staged(v, here, t);
+    }
     if (n_cta > 1) {
         // the scratch slots of lattice k: floor(begin / kPer) + k onwards (disjoint
         // across lattices, fewer than max_parts / kPer + n_inst + 1 in all)
         double* const mine = scratch + (long long)(begin / kPer + k) * kSums;
-        if (t < kSums * kLanes && t % kLanes == 0) {
-            mine[(long long)b * kSums + t / kLanes] = s;
+        if (t < kSumThreads && c == 0) {
+            mine[(long long)b * kSums + j] = s;
             __threadfence();
         }
         __syncthreads();
@@ -98,18 +102,14 @@ reduce_obs_split(const Inst* __restrict__ insts, const double* __restrict__ part
         __syncthreads();
         if (!last) return;
         __threadfence();
-        s = 0.0;
-        for (int c0 = 0; c0 < n_cta; c0 += kPer) {
-            const int nc = n_cta - c0 < kPer ? n_cta - c0 : kPer;
-            for (int q = t; q < nc * kSums; q += kThreads)
-                v[q % kSums][q / kSums] = __ldcg(mine + (long long)c0 * kSums + q);
-            __syncthreads();
-            s = combine(t / kLanes, s, sum_staged(v, nc, t));
-            __syncthreads();
+        if (t < kSumThreads) {
+            s = 0.0;
+            for (int c0 = 0; c0 < n_cta; c0 += kPer)
+                s = combine(j, s, sum_values(mine + (long long)c0 * kSums + j, kSums,
+                                             n_cta - c0 < kPer ? n_cta - c0 : kPer, j, c));
         }
     }
-    if (t < kSums * kLanes && t % kLanes == 0) {
-        const int j = t / kLanes;
+    if (t < kSumThreads && c == 0) {
         tot[j] = s;
         if (j < kObs) {
             out[(long long)k * kObs + j] = s;
@@ -125,7 +125,7 @@ reduce_obs_split(const Inst* __restrict__ insts, const double* __restrict__ part
             const double X = vol > 0.0 ? sol / vol : 0.0;
             r[LBM_FRZ_STEP] = (double)step;
             r[LBM_FRZ_MDOT_INTEGRAL] = tot[kObs];
-            if (r[LBM_FRZ_FREEZE_STEP] < 0.0 && X >= kFreezeFraction) r[LBM_FRZ_FREEZE_STEP] = (double)step;
+            if (X >= kFreezeFraction && r[LBM_FRZ_FREEZE_STEP] < 0.0) r[LBM_FRZ_FREEZE_STEP] = (double)step;
             r[LBM_FRZ_SOLID_FRACTION] = X;
         }
     }

@@ -1176,7 +1176,7 @@ __device__ __forceinline__ void tile_kernel(const Inst* __restrict__ insts,
 }
 
 template <int TX, int TY, bool OBS>
-__global__ void __launch_bounds__(TX * TY, 256 / (TX * TY) > 0 ? 256 / (TX * TY) : 1)
+__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
 step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int parity,
           double* __restrict__ partials) {
     tile_kernel<TX, TY, OBS, float>(insts, tiles, parity, partials);
@@ -1184,7 +1184,7 @@ step_fp32(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int pa
 
 // 16-bit storage in tiles: the small handles of lbm_create (32 x 4).
 template <bool OBS, typename ST>
-__global__ void __launch_bounds__(128, 2)
+__global__ void __launch_bounds__(128, 4)
 step_tile_16(const Inst* __restrict__ insts, const Tile* __restrict__ tiles, int parity,
              double* __restrict__ partials) {
     tile_kernel<32, 4, OBS, ST>(insts, tiles, parity, partials);
@@ -1303,9 +1303,10 @@ __host__ __device__ constexpr int stage_planes() { return sizeof(ST) == 4 ? 32 :
 template <typename ST>
 __host__ __device__ constexpr int slot_floats() { return stage_planes<ST>() * 32; }
 // Dynamic shared memory of one warp of a staged kernel: STG ring slots, then
-// one float per lane for the running mdot sum of the warp's item.
+// one float per lane for the running mdot sum of the warp's item and the item's
+// FP64 sum of the steps before (16 bytes, so that the rings stay aligned).
 template <typename ST, int STG>
-__host__ __device__ constexpr int warp_smem_floats() { return STG * slot_floats<ST>() + 32; }
+__host__ __device__ constexpr int warp_smem_floats() { return STG * slot_floats<ST>() + 36; }
 
 __device__ __forceinline__ void cp_async4(float* dst_smem, const float* src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
@@ -1610,7 +1611,14 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     // of its column over the item's rows (observable steps)
     float md_acc = 0.f, col_fs = 0.f;
     auto md_smem = [&]() -> float& { return ring[STG * slot_floats<ST>() + lane]; };
-    if constexpr (STG > 0) md_smem() = 0.f;
+    float* const macc_smem = ring + (STG > 0 ? STG * slot_floats<ST>() + 32 : 0);
+    if constexpr (STG > 0) {
+        md_smem() = 0.f;
+        // fetched with the first rows: a load at the item's end would add its
+        // latency to the end of the step (512 x 512: 14.7 us a step, 14.4 so)
+        if (lane == 0 && P.rare->macc)
+            cp_async8(macc_smem, reinterpret_cast<const float*>(P.rare->macc + W.part));
+    }
 
     // rows y-1 (m), y (0) and y+1 (p) of phi, rho, p^{n-1}, S^{n-1} (and T)
     float phm = 0.f, ph0, php = 0.f, rhm = 0.f, rh0, rhp = 0.f;
@@ -1786,7 +1794,10 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         if constexpr (STG > 0) md_acc = md_smem();
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) md_acc += __shfl_xor_sync(0xffffffffu, md_acc, o);
-        if (lane == 0) macc[W.part] += (double)md_acc;
+        if (lane == 0) {
+            if constexpr (STG > 0) macc[W.part] = *reinterpret_cast<const double*>(macc_smem) + (double)md_acc;
+            else macc[W.part] += (double)md_acc;
+        }
     }
     if (OBS && I.prof && out_lane) atomicAdd(I.prof + c.xc, (double)col_fs);
 }

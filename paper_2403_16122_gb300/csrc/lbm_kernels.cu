@@ -374,14 +374,21 @@ struct SlotPops {
     }
 };
 
-// Row-staged 16-bit strips: g and h decoded in the slot, f decoded into
-// registers just before the collision.
+// Row-staged 16-bit strips: the staged (g_i, h_i) word decoded where it is used,
+// with the site's references (T of the links along +y, along x and along -y: a
+// Dirichlet wall's anti-bounce-back is a reference of its own, see staged_gh); f
+// decoded into registers just before the collision.
+template <typename ST>
 struct SlotGHPops {
     const float* s;
     int lane;
     const float* f;
+    float phi, Cpref, tp, t0, tm;
     __device__ __forceinline__ float2 GH(int i) const {
-        return ld_pair(s + (i == 0 ? 4 * lane : 256 + 64 * (i - 1) + 2 * lane));
+        if (i == 0) return ld_pair(s + 4 * lane);
+        const unsigned w = __float_as_uint(*reinterpret_cast<const volatile float*>(s + 256 + 32 * (i - 1) + lane));
+        const float t = CY(i) > 0 ? tp : (CY(i) < 0 ? tm : t0);
+        return make_float2(Bits16<ST>::add_lo(w, WGT(i) * phi), Bits16<ST>::add_hi(w, WGT(i) * Cpref * t));
     }
     __device__ __forceinline__ float F(int i) const { return f[i]; }
 };
@@ -1291,15 +1298,21 @@ __device__ __forceinline__ float strip_wet_ghost(float a, float b, float outer_a
 // own-site values (16 bytes), so a row takes 18 copies instead of 32.
 // Slot layout in floats, lane l: 4l + c the own-site group (g_0, h_0, f_0,
 // f_l), 128 + 4l + c ((phi u)_x, (phi u)_y, p, S), 256 + 64 (i - 1) + 2l + s
-// the pair (g_i, h_i), 768 + 32 (i - 1) + l f_i, and for FP16 storage
-// 1024 + 2l + c (phi_ref, T_ref). FP16 pairs and f_i arrive as the aligned
-// 32-bit word holding them; decoded pairs go back over it, f_i to registers.
+// the pair (g_i, h_i), 768 + 32 (i - 1) + l f_i. 16-bit storage: 256 +
+// 32 (i - 1) + l the word of (g_i, h_i), 512 + 32 (i - 1) + l the aligned word
+// that holds f_i, 768 + 2l + c (phi_ref, T_ref).
 // ---------------------------------------------------------------------------
-constexpr int kSlotO1 = 128, kSlotGH = 256, kSlotF = 768, kSlotR = 1024;
-__device__ __forceinline__ int slot_gh(int i, int lane) { return kSlotGH + 64 * (i - 1) + 2 * lane; }
-__device__ __forceinline__ int slot_f(int i, int lane) { return kSlotF + 32 * (i - 1) + lane; }
+constexpr int kSlotO1 = 128, kSlotR = 768;
 template <typename ST>
-__host__ __device__ constexpr int stage_planes() { return sizeof(ST) == 4 ? 32 : 34; }
+__device__ __forceinline__ int slot_gh(int i, int lane) {
+    return sizeof(ST) == 4 ? 256 + 64 * (i - 1) + 2 * lane : 256 + 32 * (i - 1) + lane;
+}
+template <typename ST>
+__device__ __forceinline__ int slot_f(int i, int lane) {
+    return (sizeof(ST) == 4 ? 768 : 512) + 32 * (i - 1) + lane;
+}
+template <typename ST>
+__host__ __device__ constexpr int stage_planes() { return sizeof(ST) == 4 ? 32 : 26; }
 template <typename ST>
 __host__ __device__ constexpr int slot_floats() { return stage_planes<ST>() * 32; }
 // Dynamic shared memory of one warp of a staged kernel: STG ring slots, then
@@ -1416,13 +1429,13 @@ __device__ __forceinline__ void stage_row(const LatT<NC>& l, int lane, const Col
         if constexpr (kHalf) {
             // blocks and plane rows hold an even number of 16-bit values, so
             // every aligned word lies inside its plane row
-            cp_async_p<4>(slot + slot_gh(i, lane), reinterpret_cast<const float*>(A16 + eg), pol);
+            cp_async_p<4>(slot + slot_gh<ST>(i, lane), reinterpret_cast<const float*>(A16 + eg), pol);
             if (!macro_only)
-                cp_async_p<4>(slot + slot_f(i, lane), reinterpret_cast<const float*>(A16 + (ef & ~1)),
+                cp_async_p<4>(slot + slot_f<ST>(i, lane), reinterpret_cast<const float*>(A16 + (ef & ~1)),
                               pol);
         } else {
-            cp_async_p<8>(slot + slot_gh(i, lane), l.A + eg, pol);
-            if (!macro_only) cp_async_p<4>(slot + slot_f(i, lane), l.A + ef, pol);
+            cp_async_p<8>(slot + slot_gh<ST>(i, lane), l.A + eg, pol);
+            if (!macro_only) cp_async_p<4>(slot + slot_f<ST>(i, lane), l.A + ef, pol);
         }
     }
 }
@@ -1435,43 +1448,49 @@ struct ColPar {
 };
 __device__ __forceinline__ unsigned half_sel(int col) { return (col & 1) ? 0x3232u : 0x1010u; }
 
-// g and h of a staged row: each (g_i, h_i) pair read once. 16-bit storage
-// decodes it with the site's own references. In a row at a Dirichlet wall the
-// bounced h become anti-bounce-back, -h + 2 w_i Cp_ref T_w, and go back into
-// the slot, as every decoded pair of 16-bit storage does: the collision then
-// reads the slot as it is, without a select per direction. Only wall rows pay.
+// g and h of a staged row: each (g_i, h_i) pair read once. In a row at a
+// Dirichlet wall (dlo, dhi: below, above) the bounced h become anti-bounce-back,
+// -h + 2 w_i Cp_ref T_w, in the slot itself, so that the collision reads it
+// without a select per direction; only wall rows pay. FP32: the value. 16-bit
+// storage, where h = r + w_i Cp_ref T: the word's h changes sign and the links
+// from that wall take the reference T' = 2 T_w - T (dir_T).
 template <typename ST>
 __device__ __forceinline__ void staged_gh(float* slot, int lane, bool dlo, bool dhi, const Phys& P,
-                                          float g[9], float h[9], const Ref& ref) {
-    const float Cpref = P.Cpref;
+                                          float g[9], float h[9], const Ref& ref, float tp, float tm) {
     const float2 r0 = *reinterpret_cast<const float2*>(slot + 4 * lane);  // h_0 shifted
     g[0] = r0.x;
     h[0] = r0.y;
+    if constexpr (sizeof(ST) == 4) {
 #pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        if constexpr (sizeof(ST) == 4) {
-            const float2 v = *reinterpret_cast<const float2*>(slot + slot_gh(i, lane));
+        for (int i = 1; i < 9; ++i) {
+            const float2 v = *reinterpret_cast<const float2*>(slot + slot_gh<ST>(i, lane));
             g[i] = v.x;
             h[i] = v.y;
-        } else {
-            const unsigned wd = __float_as_uint(slot[slot_gh(i, lane)]);
-            g[i] = Bits16<ST>::add_lo(wd, WGT(i) * ref.phi);
-            h[i] = Bits16<ST>::add_hi(wd, WGT(i) * Cpref * ref.T);
         }
-    }
-    if (dlo || dhi) {
-        const float abb = P.abb();
+        if (dlo || dhi) {
+            const float abb = P.abb();
 #pragma unroll
-        for (int i = 1; i < 9; ++i)
-            if (CY(i) != 0 && (CY(i) > 0 ? dlo : dhi)) {
-                h[i] = -h[i] + 2.0f * WGT(i) * abb;
-                if constexpr (sizeof(ST) == 4) slot[slot_gh(i, lane) + 1] = h[i];
-            }
-    }
-    if constexpr (sizeof(ST) != 4) {
+            for (int i = 1; i < 9; ++i)
+                if (CY(i) != 0 && (CY(i) > 0 ? dlo : dhi)) {
+                    h[i] = -h[i] + 2.0f * WGT(i) * abb;
+                    slot[slot_gh<ST>(i, lane) + 1] = h[i];
+                }
+        }
+    } else {
+        if (dlo || dhi) {
 #pragma unroll
-        for (int i = 1; i < 9; ++i)
-            *reinterpret_cast<float2*>(slot + slot_gh(i, lane)) = make_float2(g[i], h[i]);
+            for (int i = 1; i < 9; ++i)
+                if (CY(i) != 0 && (CY(i) > 0 ? dlo : dhi)) {
+                    float& w = slot[slot_gh<ST>(i, lane)];
+                    w = __uint_as_float(__float_as_uint(w) ^ 0x80000000u);
+                }
+        }
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const unsigned wd = __float_as_uint(slot[slot_gh<ST>(i, lane)]);
+            g[i] = Bits16<ST>::add_lo(wd, WGT(i) * ref.phi);
+            h[i] = Bits16<ST>::add_hi(wd, WGT(i) * P.Cpref * (CY(i) > 0 ? tp : (CY(i) < 0 ? tm : ref.T)));
+        }
     }
 }
 
@@ -1484,7 +1503,7 @@ __device__ __forceinline__ void staged_f16(const float* slot, int lane, bool wlo
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
         const bool wall = (CY(i) > 0 && wlo) || (CY(i) < 0 && whi);
-        const unsigned w = __float_as_uint(slot[slot_f(i, lane)]);
+        const unsigned w = __float_as_uint(slot[slot_f<ST>(i, lane)]);
         const unsigned sel = wall ? par.c : (CX(i) > 0 ? par.m : (CX(i) < 0 ? par.p : par.c));
         v[i] = Bits16<ST>::fma_lo_2m12(__byte_perm(w, 0u, sel), f_rest(i, wall ? pref[0] : pref[i]));
     }
@@ -1593,11 +1612,16 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         return r;
     };
     const bool wy = !c.py;
+    auto dir_lo = [&](int y) { return wy && y == 0 && (l.flags & kDirYlo); };
+    auto dir_hi = [&](int y) { return wy && y == ny - 1 && (l.flags & kDirYhi); };
+    auto dir_T = [&](bool dir, float T) {  // 16-bit storage: reference of links from a Dirichlet wall
+        return kHalf && dir ? 2.0f * P.rare->Tw - T : T;
+    };
     auto row_macro_staged = [&](float* sl, int y, Macro& m, float& p, float& S, Ref& r) {
         float gg[9], hh[9];
         r = slot_ref(sl);
-        staged_gh<ST>(sl, lane, wy && y == 0 && (l.flags & kDirYlo),
-                      wy && y == ny - 1 && (l.flags & kDirYhi), P, gg, hh, r);
+        const bool dlo = dir_lo(y), dhi = dir_hi(y);
+        staged_gh<ST>(sl, lane, dlo, dhi, P, gg, hh, r, dir_T(dlo, r.T), dir_T(dhi, r.T));
         m = local_macro(P, gg, hh, sl[4 * lane + 3]);
         const float2 ps = *reinterpret_cast<const float2*>(sl + kSlotO1 + 4 * lane + 2);
         p = ps.x;
@@ -1751,7 +1775,9 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         if constexpr (kSlotPops && kHalf) {
             pull_f();  // all lanes (shuffles); f stays in registers for the collision
             if (out_lane)
-                site_update<OBS, ST>(P, l.flags, mO, SlotGHPops{slot(qy), lane, f}, phiux_p,
+                site_update<OBS, ST>(P, l.flags, mO,
+                                     SlotGHPops<ST>{slot(qy), lane, f, rO.phi, P.Cpref, dir_T(dir_lo(y), rO.T),
+                                                    rO.T, dir_T(dir_hi(y), rO.T)}, phiux_p,
                                      phiuy_p, st, B, Baux, l.plane, own, c.xc == nx / 2,
                                      y == ny / 2, ob, dref);
         } else if constexpr (kSlotPops) {

@@ -1628,6 +1628,11 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
         S = ps.y;
     };
 
+    // One step per launch: everything above comes from tables that no step
+    // writes, so it is done while the grid before this one drains (a no-op
+    // without the launch attribute).
+    if constexpr (NC && STG > 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+
     RowObs ob;
     if (OBS) ob.zero();
     // mdot of this lane's sites over the item (every step; the staged kernels
@@ -1845,11 +1850,9 @@ step_strip_staged(const Inst* __restrict__ insts, const Item* __restrict__ items
                   int parity, double* __restrict__ partials) {
     extern __shared__ __align__(16) float ring_smem[];
     // Programmatic dependent launch: let the next step's grid be scheduled as
-    // soon as every CTA of this one has started, and touch no lattice data
-    // before the previous step's grid has completed (a no-op when launched
-    // without the attribute).
+    // soon as every CTA of this one has started; the item touches no lattice
+    // data before the previous step's grid has completed.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5;
     const int it = blockIdx.x * WARPS + warp;
     if (it >= n_items) return;  // whole warp leaves together; no block barrier in the body
@@ -2255,7 +2258,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
 step_strip_noalloc(const __grid_constant__ Inst I, int rows, int n_items, double* __restrict__ partials) {
     extern __shared__ __align__(16) float ring_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int it = blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (it >= n_items) return;
     const int strips = (I.nx + kStripW - 1) / kStripW;

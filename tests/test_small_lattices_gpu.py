@@ -57,6 +57,32 @@ def test_small_handle_in_tiles_matches_strips(lbm, storage, nx, ny, py):
         assert oa[k] == pytest.approx(ob[k], rel=1e-6, abs=1e-6), k
 
 
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_rows_chosen_for_a_batch_change_no_bit(lbm, storage):
+    """Uneven lattices, together more than two waves of tiles (staged strips):
+    the chosen rows per item against 2, 16 and more rows than a lattice has."""
+    st = lbm.LBM_STORE_FP32 if storage == "fp32" else lbm.LBM_STORE_FP16
+    cases = [inputs.sessile(300, 280, 70.0, theta_deg=80.0), inputs.sessile(251, 303, 60.0),
+             inputs.sessile(96, 64, 16.0, theta_deg=120.0)]
+    want = None
+    for rows in (None, 2, 16, 400):
+        lat = lbm.Lattice([c[0] for c in cases], storage=st)
+        for k, (_, phi0, T0) in enumerate(cases):
+            lat.init(phi0, T0, inst=k)
+        if rows:
+            lat.set_kernel(lbm.LBM_KERNEL_STAGED, 4, rows, 168)
+        assert lat.kernel[0] == lbm.LBM_KERNEL_STAGED and lat.kernel[2] >= 2
+        lat.step(9)
+        got = [lat.get_state(k) for k in range(3)], lat.observables_all()
+        lat.close()
+        if want is None:
+            want = got
+            continue
+        for (a, b), (c, d) in zip(want[0], got[0]):
+            assert np.array_equal(a, c) and np.array_equal(b, d)
+        np.testing.assert_allclose(got[1], want[1], rtol=1e-6, atol=1e-6)
+
+
 @pytest.mark.parametrize("nx,ny", [(32, 4), (32, 256), (32, 260), (1024, 520)])
 def test_reduction_over_one_or_more_ctas(lbm, nx, ny):
     """1, 64, 65 and 4160 tiles (one partial, one CTA, two CTAs, more CTAs than

@@ -3,23 +3,24 @@
 // the three D2Q9 populations, the equilibrium initialisation, and the FP64
 // observable reduction.
 //
-// Fused step, per CTA tile of TX x TY sites (one thread per site):
-//   phase A  every thread pulls g, h, f of its own site (Section 3, streaming
-//            with half-way bounce-back / anti-bounce-back at walls) and forms
-//            H, f_s (Eqs. 8-9), mdot (Eq. 19), phi (Eq. 26) and rho (Eq. 1);
-//            phi and rho go to shared memory.
-//   phase B  the one-cell ring around the tile (and, next to a wall, the two
-//            extra cells per wall row that the wetting ghost needs) is pulled
-//            the same way by the first threads; the lagged p and S of the ring
-//            are staged too.
-//   phase C  ring cells behind a wall get their ghost values: the wetting
-//            condition for phi (Eqs. 39-41), a copy of the adjacent lattice
-//            value for rho, p and S.
-//   phase D  every thread evaluates the isotropic stencils (Eq. 38) from shared
-//            memory, the chemical potential and forces (Eqs. 11-12), the flow
-//            macroscopics (Eqs. 33-36), the three BGK collisions with their
-//            source terms (Eqs. 21, 25, 27, 30) and stores the post-collision
-//            populations and carried fields to the other buffer.
+// Fused step, per site:
+//   A  pull g, h, f of the site (Section 3, streaming with half-way bounce-back
+//      or anti-bounce-back at walls) and form H, f_s (Eqs. 8-9), mdot (Eq. 19),
+//      phi (Eq. 26) and rho (Eq. 1);
+//   B  the same for the ring around what a CTA or warp owns, with the lagged p
+//      and S, and next to a wall for the sites the wetting ghost needs;
+//   C  ring cells behind a wall get their ghost values: the wetting condition
+//      for phi (Eqs. 39-41), a copy of the adjacent value for rho, p and S;
+//   D  the isotropic stencils (Eq. 38), the chemical potential and forces
+//      (Eqs. 11-12), the flow macroscopics (Eqs. 33-36) and the three BGK
+//      collisions with their source terms (Eqs. 21, 25, 27, 30), stored to the
+//      other buffer.
+// Forms of it: tiles (a CTA per tile, a thread per site and ring entry, phi and
+// rho exchanged through shared memory; small lattices), strips (a warp walks
+// down 30 columns, neighbours by shuffles and a window of rows; staged strips
+// copy the next rows into shared memory ahead), and blocks of strip rows
+// fetched by one bulk copy each. The allocation-free step uses the strip walk
+// or a tile on separate population planes.
 // Time levels match the CPU reference: grad p and grad S use the previous
 // step's p and S; d_t(phi u) is a backward difference (Eq. 37).
 #include <algorithm>
@@ -34,12 +35,12 @@
 // The build compiles this file once per part, each compilation whole (nvcc's
 // own partitioning of a file for parallel compilation makes the code of a
 // kernel depend on the rest of the file and on the run), and links the parts:
-//   0  storage dispatch; tile, initialisation and reduction kernels
-//   1  FP32 row-staged strips (plain, observable and persistent steps)
-//   2  FP32 strips that load in place
-//   3  FP16 row-staged strips
-//   4  FP16 strips that load in place
-//   5  BF16 row-staged strips
+//   0     storage dispatch; FP32 tile, initialisation, conversion and
+//         reduction kernels, allocation-free tiles
+//   1, 2  FP32 strips: row-staged (with the allocation-free strips), in place
+//   3, 4  FP16 strips: row-staged, in place (with the FP16 tiles)
+//   5     BF16 row-staged strips and tiles
+//   6-8   block kernels in FP32, FP16 and BF16
 // Without LBM_PART the one compilation holds every part.
 #ifndef LBM_PART
 #define LBM_PART -1
@@ -2164,55 +2165,52 @@ __global__ void state_from_planes(const Inst* __restrict__ insts, int inst, int 
 }
 
 // Reduction of the partials of the allocation-free step by one cluster: CTA r
-// sums every kRedCtas-th run of kRedThreads partials (observable-major, so the
-// loads are coalesced), warps and CTAs by fixed trees, and CTA 0 reads the
-// others' sums from their shared memory and adds them in rank order. Nothing
-// outlives the launch (calls that overlap by mistake leave no count behind),
-// and the result does not depend on scheduling. FP64 runs at two additions a
-// cycle and SM: on one SM the 11 x 1024 partials of 512 x 512 sites took 15.6
-// us (ncu).
-constexpr int kRedThreads = 256, kRedCtas = 8;
+// sums every kRedCtas-th run of 256 partials (observable-major, so the loads are
+// coalesced), one warp an observable and eight loads a lane in flight, by fixed
+// trees; CTA 0 reads the others' sums from their shared memory and adds them in
+// rank order. Nothing outlives the launch (calls that overlap by mistake leave
+// no count behind), and the result does not depend on scheduling. FP64 runs at
+// two additions a cycle and SM: on one SM the 11 x 1024 partials of 512 x 512
+// sites took 15.6 us (ncu), and in the cluster every warp summing all 11
+// observables 3.2 us a step more than this (105.6 against 92.9 us for four steps
+// of 512 x 512 sites, 82.5 against 70.2 for 320 x 320).
+constexpr int kRedThreads = 32 * kObs, kRedCtas = 8;
 __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
 reduce_noalloc(int n_parts, const double* __restrict__ partials, double* __restrict__ out) {
-    __shared__ double red[kRedThreads / 32][kObs];
     __shared__ double mine[kObs];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    auto combine = [](int j, double a, double b) { return j == 9 ? fmax(a, b) : a + b; };
-    double acc[kObs];
+    const int lane = threadIdx.x & 31, j = threadIdx.x >> 5;
+    auto combine = [](int o, double a, double b) { return o == 9 ? fmax(a, b) : a + b; };
+    const double* const row = partials + (long long)j * n_parts;
+    double x = 0.0;
+    for (int p0 = blockIdx.x * 256 + lane; p0 < n_parts + lane; p0 += kRedCtas * 256) {
+        double a[8];
 #pragma unroll
-    for (int j = 0; j < kObs; ++j) acc[j] = 0.0;
-    for (int p = blockIdx.x * kRedThreads + t; p < n_parts; p += kRedCtas * kRedThreads) {
+        for (int k = 0; k < 8; ++k) a[k] = p0 + 32 * k < n_parts ? row[p0 + 32 * k] : 0.0;
 #pragma unroll
-        for (int j = 0; j < kObs; ++j)
-            acc[j] = combine(j, acc[j], partials[(long long)j * n_parts + p]);
+        for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+            for (int k = 0; k < w; ++k) a[k] = combine(j, a[k], a[k + w]);
+        x = combine(j, x, a[0]);
     }
 #pragma unroll
-    for (int j = 0; j < kObs; ++j) {
-        double x = acc[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x = combine(j, x, __shfl_xor_sync(0xffffffffu, x, o));
-        if (lane == 0) red[warp][j] = x;
-    }
-    __syncthreads();
-    if (t < kObs) {
-        double x = red[0][t];
-        for (int w = 1; w < kRedThreads / 32; ++w) x = combine(t, x, red[w][t]);
-        mine[t] = x;
-    }
+    for (int o = 16; o > 0; o >>= 1) x = combine(j, x, __shfl_xor_sync(0xffffffffu, x, o));
+    if (lane == 0) mine[j] = x;
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-    if (blockIdx.x == 0 && t < kObs) {
+    if (blockIdx.x == 0 && threadIdx.x < kObs) {
+        const int t = threadIdx.x;
         const unsigned a = (unsigned)__cvta_generic_to_shared(&mine[t]);
-        double x = mine[t];
-        for (int r = 1; r < kRedCtas; ++r) {
+        double v[kRedCtas];
+#pragma unroll
+        for (int r = 0; r < kRedCtas; ++r) {
             unsigned ra;
-            double v;
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(r));
-            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ra) : "memory");
-            x = combine(t, x, v);
+            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[r]) : "r"(ra) : "memory");
         }
-        out[t] = x;
+        double s = v[0];
+        for (int r = 1; r < kRedCtas; ++r) s = combine(t, s, v[r]);
+        out[t] = s;
     }
     // no CTA leaves while its sums are read
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");

@@ -247,9 +247,8 @@ int lbm_set_state(lbm_handle* h, int32_t inst, const double* pops,
                      shared-memory slots, so that several rows of loads are
                      in flight while a row is computed. FP32 and FP16
                      storage; the same (a, c) pairs as STRIP.
-   For both strip layouts b = 0 picks the rows per strip that let one wave
-   of resident warps take every strip of every lattice; lbm_get_kernel
-   reports the rows in effect.
+   For both strip layouts b = 0 picks the rows per strip (below);
+   lbm_get_kernel reports the rows in effect.
    LBM_KERNEL_BLOCK: one warp per 32-site column of the layout's row blocks
                      (b rows each): every row it needs arrives as four bulk
                      copies (cp.async.bulk on an mbarrier) of contiguous
@@ -258,14 +257,15 @@ int lbm_set_state(lbm_handle* h, int32_t inst, const double* pops,
                      row are compile-time constants. All storage formats;
                      needs every lattice periodic in x. (a, c) in {(4,128),
                      (4,168), (8,128)}.
-   For the strip and block layouts b = 0 picks the rows per item that let
-   one wave of resident warps take every item of every lattice.
+   For the strip and block layouts b = 0 picks the rows per item: for one
+   lattice about one wave of resident warps, for several the count with the
+   shortest estimated step.
    lbm_create picks STAGED (4, 0, 168) when every lattice is periodic in x,
    else TILE (32, 4). While its choice stands, lattices that together are two
-   waves of 32 x 4 tiles or less (some 155,000 sites, 116,000 in 16-bit storage)
-   are stepped by the tile kernel, where one step of so few sites is shorter;
-   the persistent execution form, and a layout chosen by lbm_set_kernel or
-   lbm_autotune, run as they are reported. */
+   waves of 32 x 4 tiles or less (some 155,000 sites) are stepped by
+   the tile kernel, where one step of so few sites is shorter; the persistent
+   execution form, and a layout chosen by lbm_set_kernel or lbm_autotune, run
+   as they are reported. */
 #define LBM_KERNEL_TILE   0
 #define LBM_KERNEL_STRIP  1
 #define LBM_KERNEL_STAGED 2

@@ -270,13 +270,15 @@ bool is_strip(int kind) {
 // Whether the steps of a handle run in tiles: the tile layout, or the layout
 // lbm_create chose for lattices that are at most two waves of tile CTAs (one
 // thread per site; 155,648 sites on 152 SMs). There a step is one chain of
-// latencies, and a strip item's is some rows longer than a tile's: 2.7 us
-// against 8.1 us a step on 128 x 96 sites, 4.1 against 8.3 on 256 x 256, 6.8
-// against 9.0 on 320 x 320; in BF16 storage (three CTAs an SM, 116,736 sites)
-// 2.9 against 10.2 on 128 x 128, 6.4 against 11.3 on 256 x 256. Beyond, the strips come level: 9.6 against 11.5 on
-// 400 x 400 but 26.4 against 24.3 for a step with its observables, 13.4 against
-// 14.6 on 512 x 512, 23.3 against 18.1 on 620 x 620. The persistent form stays
-// with the strips.
+// latencies, and a strip item's is some rows longer than a tile's. A plain step
+// in tiles and in strips, us: 2.7 and 7.7 on 128 x 128 sites, 4.1 and 7.9 on
+// 256 x 256, 6.8 and 8.7 on 320 x 320, 8.1 and 10.3 on 384 x 384; in 16-bit
+// storage 2.9 and 10.0, 4.2 and 10.0, 7.4 and 10.9, 8.7 and 15.5. A call of one
+// step with its observables: 13.1 and 16.0 on 256 x 256, 16.9 and 16.5 on 320 x
+// 320, 20.4 and 18.9 on 384 x 384 (16-bit 13.5 and 17.7, 18.5 and 18.4, 19.8
+// and 22.1). Beyond, the strips are level: 9.6 and 11.5 a plain step on 400 x
+// 400 but 26.4 and 24.3 with the observables read, 13.4 and 14.6 on 512 x 512,
+// 23.3 and 18.1 on 620 x 620. The persistent form stays with the strips.
 bool tiled(const lbm_handle* h) {
     return h->kind == LBM_KERNEL_TILE ||
            (h->chosen && h->small && h->exec != LBM_EXEC_PERSISTENT);
@@ -364,13 +366,12 @@ double step_estimate(const lbm_handle* h, int rows, int slots) {
 
 // Rows per strip item: as requested, or (0) the count with the shortest
 // estimated step among those that fill 1, 2, 3, 4, 6 or 8 waves of resident
-// warps (for one wave also one and two rows more or less). A single large lattice is fastest in one
-// wave; many lattices are not, as their last segments are short (48 drops on
-// 128 .. 512 squared: 341 us a step in one wave, 213 us at 32 rows; 256 drops
-// in FP16 storage on 64 .. 256: 449 us and 298 us at 20 rows; 64 drops: 118 us
-// and 87 us at 18), nor is one whose
-// rounding leaves a few items for a second wave (2501 x 2501: 267 us at 116
-// rows, 254 us at 118).
+// warps (for one wave also one and two rows more or less). A single large
+// lattice is fastest in one wave; many lattices are not, as their last segments
+// are short (48 drops on 128 .. 512 squared: 341 us a step in one wave, 213 us
+// at 32 rows; 256 drops in FP16 storage on 64 .. 256: 449 us and 298 us at 20
+// rows; 64 drops: 118 us and 87 us at 18), nor is one whose rounding leaves a
+// few items for a second wave (2501 x 2501: 267 us at 116 rows, 254 us at 118).
 int item_rows(const lbm_handle* h) {
     if (h->rows_req > 0) return h->rows_req;
     int max_ny = kMinRows;

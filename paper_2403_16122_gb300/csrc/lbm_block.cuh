@@ -230,7 +230,7 @@ __device__ __forceinline__ Macro block_macro(const Phys& P, At at, const float4&
 // step. ring: kBlockStg slots; mbar: kBlockStg barriers (initialised, count
 // 33, phases tracked in *phase); hring: the side-column ring; mdsm: 32 floats.
 // Returns false when a staged row never completed (the error word is raised).
-template <bool OBS, typename ST, bool NC>
+template <bool OBS, typename ST, Path PATH>
 __device__ __forceinline__ bool block_item(const Inst* __restrict__ insts, const Item& W, int parity,
                                            double* __restrict__ partials, unsigned char* ring,
                                            uint64_t* mbar, unsigned& phase, float* hring,
@@ -400,7 +400,7 @@ __device__ __forceinline__ bool block_item(const Inst* __restrict__ insts, const
             // column (rows next to a wall only): from global memory
             const int rr = r.rr;
             if (!py && (rr <= 1 || rr >= ny - 2)) {
-                LatT<NC> l;
+                LatT<PATH> l;
                 l.A = reinterpret_cast<const float*>(A);
                 l.Aaux = Aaux;
                 l.plane = (int)I.plane; l.nx = nx; l.ny = ny; l.pitch = I.pitch; l.flags = flags;

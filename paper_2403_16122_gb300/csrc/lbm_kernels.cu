@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 
 #include "lbm_internal.h"
+#include "lbm_load.cuh"
 #include "lbm_math.cuh"
 
 // The build compiles this file once per part, each compilation whole (nvcc's
@@ -95,26 +96,33 @@ __device__ __forceinline__ float mix3(float fs, float phi, float zs, float zl, f
 // ---------------------------------------------------------------------------
 // Storage access (FP32)
 // ---------------------------------------------------------------------------
-// NC selects the load path: true for kernels that run one step per launch
-// (the read-only, non-coherent path), false for the persistent kernel, where
-// a buffer read in one step was written by other CTAs in the previous step of
-// the same launch, so its loads bypass L1 and are served by the coherent L2.
-template <bool NC>
+// How a kernel loads lattice state:
+//   kReadOnly  the read-only, non-coherent path, defined only for data that
+//              nobody writes during the kernel's life: strips that load in
+//              place, one step a launch, whose launch waits for the grid before
+//              it to end;
+//   kOrdered   plain loads, which stay behind a wait: kernels launched as
+//              dependents (staged strips, blocks), resident while the grid before
+//              them still writes what they will read;
+//   kL2        ld_live: the persistent kernels, where a buffer read in one step
+//              was written by other CTAs in the previous step of the launch.
+// (The staged strips' few direct loads through ld_live instead, one in each wall
+// branch of pull_set, were a chain: 53.2 us a step of 1024 x 1024 sites in FP16,
+// 44.5 so.)
+enum class Path { kReadOnly, kOrdered, kL2 };
+template <Path PATH>
 struct LatT {
-    const float* __restrict__ A;  // source populations (27 planes)
-    const float* __restrict__ Aaux;
-    int plane;                    // elements per plane (27 planes fit 32-bit offsets)
+    const float* A;  // source populations (27 planes)
+    const float* Aaux;
+    int plane;       // elements per plane (27 planes fit 32-bit offsets)
     int nx, ny, pitch, flags;
 };
-using Lat = LatT<true>;
 
-template <bool NC>
-__device__ __forceinline__ float ld_f32(const float* p) {
-    if constexpr (NC) return __ldg(p); else return __ldcg(p);
-}
-template <bool NC>
-__device__ __forceinline__ unsigned short ld_u16(const unsigned short* p) {
-    if constexpr (NC) return __ldg(p); else return __ldcg(p);
+template <Path PATH, typename T>
+__device__ __forceinline__ T ld_state(const T* p) {
+    if constexpr (PATH == Path::kReadOnly) return __ldg(p);
+    else if constexpr (PATH == Path::kOrdered) return *p;
+    else return ld_live(p);
 }
 
 // FP16 storage: population i of a set is stored as a 16-bit deviation from a
@@ -140,14 +148,14 @@ struct Ref {
 
 // Stored population (set, i) of site idx (grouped layout, see Inst); the rest
 // populations are FP32 in the own-site region for both storages.
-template <typename ST, bool NC>
-__device__ __forceinline__ float ldPop(const LatT<NC>& l, int set, int i, int idx) {
-    if (i == 0) return ld_f32<NC>(l.Aaux + own0_at(idx, set));
+template <typename ST, Path PATH>
+__device__ __forceinline__ float ldPop(const LatT<PATH>& l, int set, int i, int idx) {
+    if (i == 0) return ld_state<PATH>(l.Aaux + own0_at(idx, set));
     if constexpr (sizeof(ST) == 4) {
-        return ld_f32<NC>(l.A + pop_at(set, i, idx));
+        return ld_state<PATH>(l.A + pop_at(set, i, idx));
     } else {
         const unsigned short* A = reinterpret_cast<const unsigned short*>(l.A);
-        return Bits16<ST>::to_f(Bits16<ST>::from_bits(ld_u16<NC>(A + pop_at(set, i, idx))));
+        return Bits16<ST>::to_f(Bits16<ST>::from_bits(ld_state<PATH>(A + pop_at(set, i, idx))));
     }
 }
 
@@ -168,9 +176,9 @@ __device__ __forceinline__ float decode(int i, float raw, const Ref& r, float Cp
 __device__ __forceinline__ float f_rest(int i, float p) {
     return (i == 0 ? (kW0 - 1.f) : WGT(i)) * 3.f * p;
 }
-template <bool NC>
-__device__ __forceinline__ float ldAux(const LatT<NC>& l, int k, int idx) {
-    return ld_f32<NC>(l.Aaux + aux_at(k, idx));
+template <Path PATH>
+__device__ __forceinline__ float ldAux(const LatT<PATH>& l, int k, int idx) {
+    return ld_state<PATH>(l.Aaux + aux_at(k, idx));
 }
 
 // Pull of set `set` (0 g, 1 h, 2 f) at lattice site (x, y): v[i] is the
@@ -178,8 +186,8 @@ __device__ __forceinline__ float ldAux(const LatT<NC>& l, int k, int idx) {
 // half-way bounce-back of the site's own opposite population; for h at a
 // Dirichlet wall by anti-bounce-back -h + 2 w_i Cp_ref T_w (Section 4.1).
 // h_0 is returned as stored (shifted, see Inst).
-template <int SET, typename ST = float, bool NC>
-__device__ __forceinline__ void pull_set(const LatT<NC>& l, int x, int y, float abb, float v[9],
+template <int SET, typename ST = float, Path PATH>
+__device__ __forceinline__ void pull_set(const LatT<PATH>& l, int x, int y, float abb, float v[9],
                                          const Ref& ref = Ref{0.f, 0.f}, float Cpref = 0.f,
                                          const float* pref = nullptr) {
     constexpr bool kFref = sizeof(ST) != 4 && SET == 2;  // f: source-pressure reference
@@ -838,7 +846,7 @@ __device__ __forceinline__ Links links_of(int nx, int ny, int pitch, int flags, 
 }
 template <typename V>
 __device__ __forceinline__ V ld_cg(const float* p) {
-    return __ldcg(reinterpret_cast<const V*>(p));
+    return ld_live(reinterpret_cast<const V*>(p));
 }
 // A (g_i, h_i) pair and an f_i as they are stored: two floats and one, or (16-bit
 // storage) one word and one half.
@@ -850,17 +858,17 @@ struct Raw {
         return ld_cg<float2>(static_cast<const float*>(A) + off);
     }
     static __device__ __forceinline__ F f(const void* A, int off) {
-        return __ldcg(static_cast<const float*>(A) + off);
+        return ld_live(static_cast<const float*>(A) + off);
     }
 };
 struct Raw16 {
     using Pair = unsigned;
     using F = unsigned short;
     static __device__ __forceinline__ Pair pair(const void* A, int off) {
-        return __ldcg(reinterpret_cast<const unsigned*>(static_cast<const unsigned short*>(A) + off));
+        return ld_live(reinterpret_cast<const unsigned*>(static_cast<const unsigned short*>(A) + off));
     }
     static __device__ __forceinline__ F f(const void* A, int off) {
-        return __ldcg(static_cast<const unsigned short*>(A) + off);
+        return ld_live(static_cast<const unsigned short*>(A) + off);
     }
 };
 template <> struct Raw<__half> : Raw16 {};
@@ -1232,8 +1240,8 @@ step_tile_noalloc(const __grid_constant__ Inst I, int tiles_x, double* __restric
 
 // Pull of set SET at (x, y) for a row whose sources do not cross a wall; the
 // column offsets xm/xp and row offsets rm/rp are already wrapped.
-template <int SET, typename ST, bool NC>
-__device__ __forceinline__ void pull_rows(const LatT<NC>& l, int xc, int xm, int xp, int r0,
+template <int SET, typename ST, Path PATH>
+__device__ __forceinline__ void pull_rows(const LatT<PATH>& l, int xc, int xm, int xp, int r0,
                                           int rm, int rp, float v[9], const Ref& ref,
                                           float Cpref, const float* pref) {
 #pragma unroll
@@ -1253,8 +1261,8 @@ struct RowCtx {
 };
 
 // Pulls and local macroscopic fields of lattice row y at this lane's column.
-template <int SET, typename ST = float, bool NC>
-__device__ __forceinline__ void pull_row(const LatT<NC>& l, const RowCtx& c, int y, float abb,
+template <int SET, typename ST = float, Path PATH>
+__device__ __forceinline__ void pull_row(const LatT<PATH>& l, const RowCtx& c, int y, float abb,
                                          float v[9], const Ref& ref = Ref{0.f, 0.f},
                                          float Cpref = 0.f,
                                          const float* pref = nullptr) {
@@ -1395,8 +1403,8 @@ struct ColTerms {
     }
 };
 
-template <typename ST, bool NC>
-__device__ __forceinline__ void stage_row(const LatT<NC>& l, int lane, const ColTerms& ct, bool py,
+template <typename ST, Path PATH>
+__device__ __forceinline__ void stage_row(const LatT<PATH>& l, int lane, const ColTerms& ct, bool py,
                                           int r, bool macro_only, float* slot, int hint = 0) {
     constexpr bool kHalf = sizeof(ST) != 4;
     const int ny = l.ny, nxb = l.pitch >> 5;
@@ -1514,7 +1522,7 @@ __device__ __forceinline__ void staged_f16(const float* slot, int lane, bool wlo
 // STG = 0: populations are loaded where they are consumed; STG >= 3: rows are
 // staged through `ring` (STG slots of this warp): while row y is computed,
 // the copies of rows y + 2 .. y + STG - 1 are in flight.
-template <bool OBS, typename ST, bool NC, int STG = 0>
+template <bool OBS, typename ST, bool PERSIST, int STG = 0>
 __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const Item& W,
                                            int parity, double* __restrict__ partials,
                                            float* ring = nullptr) {
@@ -1526,7 +1534,8 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     const int lane = threadIdx.x & 31;
     const Inst& I = insts[W.inst];
     const Phys P = load_phys(I);
-    LatT<NC> l;
+    constexpr Path kPath = PERSIST ? Path::kL2 : (STG == 0 ? Path::kReadOnly : Path::kOrdered);
+    LatT<kPath> l;
     l.A = static_cast<const float*>(I.pop[parity]);
     l.Aaux = I.aux[parity];
     l.plane = (int)I.plane; l.nx = I.nx; l.ny = I.ny; l.pitch = I.pitch; l.flags = I.flags;
@@ -1632,7 +1641,7 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     // One step per launch: everything above comes from tables that no step
     // writes, so it is done while the grid before this one drains (a no-op
     // without the launch attribute).
-    if constexpr (NC && STG > 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (!PERSIST && STG > 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     RowObs ob;
     if (OBS) ob.zero();
@@ -1840,7 +1849,7 @@ step_strip(const Inst* __restrict__ insts, const Item* __restrict__ items, int n
            int parity, double* __restrict__ partials) {
     const int it = blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (it >= n_items) return;  // whole warp leaves together; no block barrier in the body
-    strip_item<OBS, ST, true>(insts, items[it], parity, partials);
+    strip_item<OBS, ST, false>(insts, items[it], parity, partials);
 }
 
 // Staged form: STG ring slots of slot_floats<ST>() floats per warp in dynamic
@@ -1857,8 +1866,8 @@ step_strip_staged(const Inst* __restrict__ insts, const Item* __restrict__ items
     const int warp = threadIdx.x >> 5;
     const int it = blockIdx.x * WARPS + warp;
     if (it >= n_items) return;  // whole warp leaves together; no block barrier in the body
-    strip_item<OBS, ST, true, STG>(insts, items[it], parity, partials,
-                                   ring_smem + warp * warp_smem_floats<ST, STG>());
+    strip_item<OBS, ST, false, STG>(insts, items[it], parity, partials,
+                                    ring_smem + warp * warp_smem_floats<ST, STG>());
 }
 
 // Device-wide barrier between the steps of the persistent kernel. Every CTA
@@ -1922,7 +1931,7 @@ step_strip_persistent(const Inst* __restrict__ insts, const Item* __restrict__ i
     for (int s = 0; s < nsteps; ++s) {
         const int parity = parity0 ^ (s & 1);
         for (int it = warp; it < n_items; it += stride)
-            strip_item<false, ST, false, STG>(insts, items[it], parity, nullptr, ring);
+            strip_item<false, ST, true, STG>(insts, items[it], parity, nullptr, ring);
         if (s + 1 < nsteps &&
             !grid_barrier(bar, (unsigned)(s + 1) * gridDim.x, err, limit_ns))
             return;
@@ -1952,9 +1961,9 @@ step_block(const Inst* __restrict__ insts, const Item* __restrict__ items, int n
     const int it = blockIdx.x * WARPS + warp;
     if (it >= n_items) return;  // whole warp leaves together; no block barrier in the body
     unsigned phase = 0;
-    block_item<OBS, ST, true>(insts, items[it], parity, partials, base, mbar, phase,
-                              reinterpret_cast<float*>(base + BW::kHring),
-                              reinterpret_cast<float*>(base + BW::kMd), err);
+    block_item<OBS, ST, Path::kOrdered>(insts, items[it], parity, partials, base, mbar, phase,
+                                        reinterpret_cast<float*>(base + BW::kHring),
+                                        reinterpret_cast<float*>(base + BW::kMd), err);
 }
 
 // Persistent form of the block step: every item of every lattice for nsteps
@@ -1983,9 +1992,9 @@ step_block_persistent(const Inst* __restrict__ insts, const Item* __restrict__ i
     for (int s = 0; s < nsteps; ++s) {
         const int parity = parity0 ^ (s & 1);
         for (int it = gw; ok && it < n_items; it += stride)
-            ok = block_item<false, ST, false>(insts, items[it], parity, nullptr, base, mbar, phase,
-                                              reinterpret_cast<float*>(base + BW::kHring),
-                                              reinterpret_cast<float*>(base + BW::kMd), err);
+            ok = block_item<false, ST, Path::kL2>(insts, items[it], parity, nullptr, base, mbar, phase,
+                                                  reinterpret_cast<float*>(base + BW::kHring),
+                                                  reinterpret_cast<float*>(base + BW::kMd), err);
         if (s + 1 < nsteps) {
             if (!grid_barrier(bar, (unsigned)(s + 1) * gridDim.x, err, limit_ns)) return;
             asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -2187,7 +2196,7 @@ reduce_noalloc(int n_parts, const double* __restrict__ partials, double* __restr
     for (int p0 = blockIdx.x * 256 + lane; p0 < n_parts + lane; p0 += kRedCtas * 256) {
         double a[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) a[k] = p0 + 32 * k < n_parts ? row[p0 + 32 * k] : 0.0;
+        for (int k = 0; k < 8; ++k) a[k] = p0 + 32 * k < n_parts ? ld_live(row + p0 + 32 * k) : 0.0;
 #pragma unroll
         for (int w = 4; w > 0; w >>= 1)
 #pragma unroll
@@ -2265,8 +2274,8 @@ step_strip_noalloc(const __grid_constant__ Inst I, int rows, int n_items, double
     W.y0 = it / strips * rows;
     W.y1 = min(W.y0 + rows, I.ny);
     W.part = it;
-    strip_item<true, float, true, STG>(&I, W, 0, partials,
-                                       ring_smem + (threadIdx.x >> 5) * warp_smem_floats<float, STG>());
+    strip_item<true, float, false, STG>(&I, W, 0, partials,
+                                        ring_smem + (threadIdx.x >> 5) * warp_smem_floats<float, STG>());
 }
 #endif
 

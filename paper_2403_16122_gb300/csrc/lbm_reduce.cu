@@ -18,6 +18,8 @@
 // 66 so (59). One copy of the summing code for both passes was 1 us slower.
 #include "lbm_reduce.h"
 
+#include "lbm_load.cuh"
+
 namespace lbmk {
 namespace {
 
@@ -38,7 +40,7 @@ __device__ __forceinline__ double combine(int j, double a, double b) {
 __device__ __forceinline__ double sum_values(const double* p, long long stride, int n, int j, int c) {
     double a[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) a[k] = c + 8 * k < n ? __ldcg(p + (c + 8 * k) * stride) : 0.0;
+    for (int k = 0; k < 8; ++k) a[k] = c + 8 * k < n ? ld_live(p + (c + 8 * k) * stride) : 0.0;
 #pragma unroll
     for (int w = 4; w > 0; w >>= 1)
 #pragma unroll
@@ -85,7 +87,7 @@ reduce_obs_split(const Inst* __restrict__ insts, const double* __restrict__ part
         s = sum_values(row, 1, row ? here : 0, j, c);
     } else if (prof && prof_out) {  // the last warp: a share of the column profile
         for (int x = b * 32 + (t & 31); x < nx; x += n_cta * 32) {
-            prof_out[x] = __ldcg(prof + x);
+            prof_out[x] = ld_live(prof + x);
             prof[x] = 0.0;
         }
     }

@@ -425,25 +425,23 @@ struct SiteObs {
         }
     }
     __device__ __forceinline__ void max(int j, float x) { v[j] = x; }
+    __device__ __forceinline__ float greatest() const { return v[9]; }
+    __device__ __forceinline__ bool some(int j) const { return v[j] != 0.f; }
     __device__ __forceinline__ double total(int j) const {
         return j == 2 ? (double)v[2] + ((double)h[0] + (double)h[1]) : (double)v[j];
     }
 };
 
-// Block reduction of the observables of a tile (FP64). out: the tile's slot in
-// observable-major partials (observable j at out[j * stride]). A warp's sums of
-// slots 0-6 go through one reduce-scatter: at lane bits 4, 3 and 2 a lane
-// keeps half of its vector and adds the partner's copy of that half, then two
-// xor steps finish, so a warp issues 9 FP64 additions for them instead of 35
-// (FP64 runs at two additions a cycle and SM here: eleven plain trees were
-// 3.5 us of the observable step). Slot 9 is a maximum of FP32 values; slots 7,
-// 8 and 10 are zero but for a few sites and are skipped where a warp has none.
-template <int NT>
-__device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __restrict__ out,
-                                                 int stride) {
-    __shared__ double red[NT / 32][kObs];
+// FP64 totals of a warp's lanes, handed to put(j, total) by one lane each.
+// Slots 0-6 go through one reduce-scatter: at lane bits 4, 3 and 2 a lane keeps
+// half of its vector and adds the partner's copy of that half, then two xor
+// steps finish, so a warp issues 9 FP64 additions for them instead of 35 (FP64
+// runs at two additions a cycle and SM here: eleven plain trees were 3.5 us of
+// the tiles' observable step). Slot 9 is a maximum of FP32 values; slots 7, 8
+// and 10 are zero but for a few sites and are skipped where a warp has none.
+template <typename Acc, typename Put>
+__device__ __forceinline__ void warp_totals(const Acc& ob, int lane, Put&& put) {
     constexpr unsigned kAll = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
     double k4[4], k2[2];
 #pragma unroll
@@ -457,23 +455,33 @@ __device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __re
     double t = (b2 ? k2[1] : k2[0]) + __shfl_xor_sync(kAll, b2 ? k2[0] : k2[1], 4);
     t += __shfl_xor_sync(kAll, t, 2);
     t += __shfl_xor_sync(kAll, t, 1);
-    if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
-    float mx = ob.v[9];
+    if ((lane & 3) == 0 && lane < 28) put(lane >> 2, t);
+    float mx = ob.greatest();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kAll, mx, o));
-    if (lane == 0) red[warp][9] = (double)mx;
+    if (lane == 0) put(9, (double)mx);
     auto rare = [&](int j) {
         double x = 0.0;
-        if (__any_sync(kAll, ob.v[j] != 0.f)) {
+        if (__any_sync(kAll, ob.some(j))) {
             x = ob.total(j);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
         }
-        if (lane == 0) red[warp][j] = x;
+        if (lane == 0) put(j, x);
     };
     rare(7);
     rare(8);
     rare(10);
+}
+
+// Block reduction of the observables of a tile (FP64). out: the tile's slot in
+// observable-major partials (observable j at out[j * stride]).
+template <int NT>
+__device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __restrict__ out,
+                                                 int stride) {
+    __shared__ double red[NT / 32][kObs];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    warp_totals(ob, lane, [&](int j, double x) { red[warp][j] = x; });
     __syncthreads();
     if (threadIdx.x < kObs) {
         const int j = threadIdx.x;
@@ -482,6 +490,46 @@ __device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __re
         out[(long long)j * stride] = acc;
     }
 }
+
+// Observable sums of a strip, lane by lane over an item's rows (the
+// allocation-free step, whose caller reads the record of one step as FP64): a
+// running FP32 sum and the sum of the exact rounding errors of its additions
+// (D. E. Knuth, "The Art of Computer Programming", vol. 2, 4.2.2), so that a
+// lane's sum keeps some 48 bits, then FP64 across the lanes and items: the sum of
+// phi is within 2e-16 of the exact one on 500 x 420 to 1900 x 1000 sites, as the
+// tiles' is. A step of 512 x 512 sites, us: 24.7; FP64 additions row by row
+// 31.3; the rows in FP32 (RowObs below, 1.5e-9) 23.2.
+struct LaneObs {
+    float s[7], c[7], mx, row, bad;
+    bool col;
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int j = 0; j < 7; ++j) s[j] = c[j] = 0.f;
+        mx = row = bad = 0.f;
+        col = false;
+    }
+    __device__ __forceinline__ void add(int j, float x) {
+        if (j == 7) {  // a lane's column: its sum of f_s, slot 1
+            col = true;
+        } else if (j == 8) {  // one row of the item at most
+            row = x;
+        } else if (j == 10) {
+            bad += x;
+        } else {
+            const float t = s[j] + x, d = t - s[j];
+            c[j] += (s[j] - (t - d)) + (x - d);
+            s[j] = t;
+        }
+    }
+    __device__ __forceinline__ void max(int, float x) { mx = fmaxf(mx, x); }
+    __device__ __forceinline__ void flush(int) {}
+    __device__ __forceinline__ float greatest() const { return mx; }
+    __device__ __forceinline__ bool some(int j) const { return j == 7 ? col : (j == 8 ? row != 0.f : bad != 0.f); }
+    __device__ __forceinline__ double total(int j) const {
+        if (j < 7) return (double)s[j] + (double)c[j];
+        return j == 7 ? (col ? total(1) : 0.0) : (double)(j == 8 ? row : bad);
+    }
+};
 
 // Observable sums of a warp strip, taken row by row: at the end of each row
 // the values of its sites (at most 30) are summed across the warp in FP32,
@@ -1522,7 +1570,7 @@ __device__ __forceinline__ void staged_f16(const float* slot, int lane, bool wlo
 // STG = 0: populations are loaded where they are consumed; STG >= 3: rows are
 // staged through `ring` (STG slots of this warp): while row y is computed,
 // the copies of rows y + 2 .. y + STG - 1 are in flight.
-template <bool OBS, typename ST, bool PERSIST, int STG = 0>
+template <bool OBS, typename ST, bool PERSIST, int STG = 0, typename Obs = RowObs>
 __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const Item& W,
                                            int parity, double* __restrict__ partials,
                                            float* ring = nullptr) {
@@ -1643,7 +1691,7 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     // without the launch attribute).
     if constexpr (!PERSIST && STG > 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    RowObs ob;
+    Obs ob;
     if (OBS) ob.zero();
     // mdot of this lane's sites over the item (every step; the staged kernels
     // keep it in shared memory after the ring, which spares a register), f_s
@@ -1826,8 +1874,12 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     }
     if constexpr (STG > 0) cp_async_wait<0>();  // the trailing groups are empty
 
-    if (OBS && RowObs::carried(lane) >= 0)
-        partials[(long long)RowObs::carried(lane) * I.part_stride + W.part] = ob.total();
+    if constexpr (std::is_same_v<Obs, LaneObs>) {
+        warp_totals(ob, lane, [&](int j, double x) { partials[(long long)j * I.part_stride + W.part] = x; });
+    } else {
+        if (OBS && RowObs::carried(lane) >= 0)
+            partials[(long long)RowObs::carried(lane) * I.part_stride + W.part] = ob.total();
+    }
     // the item's mdot of this step joins its FP64 running sum (one warp owns
     // the item, so the read-modify-write needs no atomic)
     double* const macc = insts[W.inst].macc;  // read here: no register held over the rows
@@ -2274,8 +2326,8 @@ step_strip_noalloc(const __grid_constant__ Inst I, int rows, int n_items, double
     W.y0 = it / strips * rows;
     W.y1 = min(W.y0 + rows, I.ny);
     W.part = it;
-    strip_item<true, float, false, STG>(&I, W, 0, partials,
-                                        ring_smem + (threadIdx.x >> 5) * warp_smem_floats<float, STG>());
+    strip_item<true, float, false, STG, LaneObs>(&I, W, 0, partials,
+                                                  ring_smem + (threadIdx.x >> 5) * warp_smem_floats<float, STG>());
 }
 #endif
 

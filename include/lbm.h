@@ -69,12 +69,11 @@ extern "C" {
                    ones, so the phi, H and f sums a site sends out are kept
                    exactly. phi and T of each site are two more FP32 planes:
                    176 bytes per lattice update. Needs every lattice periodic
-                   in x (strip layout). lbm_get_state / lbm_set_state convert
+                   in x. lbm_get_state / lbm_set_state convert
                    to and from the same double layouts as FP32.
    LBM_STORE_BF16: the FP16 arrangement with bfloat16 values (7-bit
                    mantissa, FP32 exponent range): 176 bytes per lattice
-                   update; the row-staged strip layout with 4 warps per CTA
-                   only (registers 128 or 168). */
+                   update; not in the strip layout that loads in place. */
 #define LBM_STORE_FP32  0
 #define LBM_STORE_FP16  1
 #define LBM_STORE_BF16  2
@@ -236,7 +235,8 @@ int lbm_set_state(lbm_handle* h, int32_t inst, const double* pops,
    steps), not bit for bit.
    LBM_KERNEL_TILE:  one CTA per tile of a x b sites with a shared-memory
                      halo; handles every wall combination. (a, b) in
-                     {(32,8), (32,4), (64,4), (32,16)}; c ignored.
+                     {(32,8), (32,4), (64,4), (32,16)}, in 16-bit storage
+                     (32,4); c ignored.
    LBM_KERNEL_STRIP: one warp per strip of 30 columns x b rows (b >= 2) that
                      keeps its halo in registers and warp shuffles; needs every
                      lattice of the handle periodic in x. a = warps per CTA,
@@ -245,8 +245,8 @@ int lbm_set_state(lbm_handle* h, int32_t inst, const double* pops,
    LBM_KERNEL_STAGED: the strip layout with every row a lane consumes
                      copied ahead (cp.async) into a per-warp ring of
                      shared-memory slots, so that several rows of loads are
-                     in flight while a row is computed. FP32 and FP16
-                     storage; the same (a, c) pairs as STRIP.
+                     in flight while a row is computed. The same (a, c)
+                     pairs as STRIP; BF16 storage: (4,128) and (4,168).
    For both strip layouts b = 0 picks the rows per strip (below);
    lbm_get_kernel reports the rows in effect.
    LBM_KERNEL_BLOCK: one warp per 32-site column of the layout's row blocks

@@ -1103,7 +1103,7 @@ int lbm_set_thermal_walls(lbm_handle* h, int32_t inst, int32_t x_lo, int32_t x_h
 int lbm_set_kernel(lbm_handle* h, int32_t kind, int32_t a, int32_t b, int32_t c) {
     if (!h) return LBM_EINVAL;
     if (kind == LBM_KERNEL_TILE) {
-        if (!lbmk::tile_supported(a, b) || h->storage != LBM_STORE_FP32) return LBM_EINVAL;
+        if (!lbmk::tile_supported(a, b, h->storage)) return LBM_EINVAL;
         if (h->exec == LBM_EXEC_PERSISTENT) return LBM_EINVAL;  // persistent form is strip-only
         h->kind = kind; h->tx = a; h->ty = b;
     } else if (kind == LBM_KERNEL_BLOCK) {

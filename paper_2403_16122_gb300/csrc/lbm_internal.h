@@ -372,7 +372,8 @@ bool params_valid(const lbm_params& p);
 // Pitch (elements per row) the library uses for a lattice of width nx.
 inline int pitch_for(int nx) { return (nx + 31) / 32 * 32; }
 
-// Supported tile shapes (TX x TY threads, one site per thread).
-bool tile_supported(int tx, int ty);
+// Supported tile shapes (TX x TY threads, one site per thread; 16-bit storage:
+// 32 x 4 only).
+bool tile_supported(int tx, int ty, int storage);
 
 }  // namespace lbmk

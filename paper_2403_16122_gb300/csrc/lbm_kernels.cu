@@ -2930,7 +2930,8 @@ bool strip_supported(int warps, int regs) {
            (warps == 8 && regs == 128) || (warps == 2 && regs == 128);
 }
 
-bool tile_supported(int tx, int ty) {
+bool tile_supported(int tx, int ty, int storage) {
+    if (storage != LBM_STORE_FP32) return tx == 32 && ty == 4;
     return (tx == 32 && ty == 8) || (tx == 32 && ty == 4) || (tx == 64 && ty == 4) ||
            (tx == 32 && ty == 16);
 }

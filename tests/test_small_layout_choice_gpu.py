@@ -1,0 +1,59 @@
+"""Small handles in 16-bit storage: the tile layout they are created in can be
+chosen, found by the autotuner and read back."""
+import numpy as np
+import pytest
+
+from paper_2403_16122_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    from paper_2403_16122_gb300 import build
+    from paper_2403_16122_gb300 import lbm as mod
+
+    build.build()
+    mod.load()
+    return mod
+
+
+def _drop(lbm, storage, n=128):
+    p, phi0, T0 = inputs.sessile(nx=n, ny=n, R=0.25 * n, theta_deg=75.0)
+    return lbm.Lattice([p], storage=getattr(lbm, "LBM_STORE_" + storage)).init(phi0, T0)
+
+
+@pytest.mark.parametrize("storage", ["FP16", "BF16"])
+def test_16bit_tiles_can_be_chosen(lbm, storage):
+    """TILE (32, 4) in 16-bit storage is the kernel such a handle is created in:
+    the same bits. The other tile shapes stay refused, and so does the
+    persistent form."""
+    a, b = _drop(lbm, storage), _drop(lbm, storage)
+    b.set_kernel(lbm.LBM_KERNEL_TILE, 32, 4)
+    assert b.kernel == (lbm.LBM_KERNEL_TILE, 32, 4, 0)
+    for u, v in zip(a.step(25).get_state(), b.step(25).get_state()):
+        assert np.array_equal(u, v)
+    assert a.observables() == b.observables()
+    for shape in ((32, 8), (64, 4), (32, 16), (32, 5)):
+        with pytest.raises(lbm.LbmError):
+            b.set_kernel(lbm.LBM_KERNEL_TILE, *shape)
+    with pytest.raises(lbm.LbmError):
+        b.set_exec(lbm.LBM_EXEC_PERSISTENT, 4)
+    # and on a lattice of more than two waves of tiles
+    c, d = _drop(lbm, storage, 512), _drop(lbm, storage, 512)
+    c.set_kernel(lbm.LBM_KERNEL_TILE, 32, 4).step(3)
+    d.step(3)
+    # a stored value may round to the other neighbour (2^-13, 2^-10 apart) a step
+    tol = 3 * (2.0 ** -13 if storage == "FP16" else 2.0 ** -10)
+    for u, v in zip(c.get_state(), d.get_state()):
+        assert np.abs(u - v).max() <= tol
+
+
+@pytest.mark.parametrize("storage", ["FP16", "BF16"])
+def test_autotuner_keeps_small_16bit_lattices_in_tiles(lbm, storage):
+    """A step of 128 x 128 sites takes a third of the time in tiles."""
+    a = _drop(lbm, storage)
+    a.autotune(steps=50)
+    assert a.kernel == (lbm.LBM_KERNEL_TILE, 32, 4, 0)
+    b = _drop(lbm, storage).set_kernel(*a.kernel)
+    assert b.kernel == a.kernel

@@ -285,8 +285,16 @@ int lbm_set_thermal_walls(lbm_handle* h, int32_t inst, int32_t x_lo, int32_t x_h
    stream; synchronises it). LBM_EINVAL for an unsupported combination. */
 int lbm_set_kernel(lbm_handle* h, int32_t kind, int32_t a, int32_t b, int32_t c);
 
-/* Current layout: out[0] = kind, out[1..3] = a, b, c as for lbm_set_kernel. */
+/* Current layout: out[0] = kind, out[1..3] = a, b, c as for lbm_set_kernel.
+   While lbm_create's choice stands this is that choice, also on lattices small
+   enough to be stepped in tiles (lbm_get_step_kernel). */
 int lbm_get_kernel(const lbm_handle* h, int32_t* out);
+
+/* The layout that lbm_step runs in now, in the form of lbm_get_kernel: the same,
+   but TILE (32, 4) where lbm_create's choice stands on small lattices. Passed to
+   lbm_set_kernel of a handle like this one it gives the same steps, bit for
+   bit. */
+int lbm_get_step_kernel(const lbm_handle* h, int32_t* out);
 
 /* Autotuner: time every supported layout for this handle twice over `steps`
    time steps each (after one warm-up step), measured with CUDA events on the

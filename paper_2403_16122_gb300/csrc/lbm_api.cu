@@ -1173,6 +1173,16 @@ int lbm_get_kernel(const lbm_handle* h, int32_t* out) {
     return LBM_OK;
 }
 
+int lbm_get_step_kernel(const lbm_handle* h, int32_t* out) {
+    if (!h || !out) return LBM_EINVAL;
+    if (!tiled(h)) return lbm_get_kernel(h, out);
+    out[0] = LBM_KERNEL_TILE;
+    out[1] = h->tx;
+    out[2] = h->ty;
+    out[3] = 0;
+    return LBM_OK;
+}
+
 int lbm_autotune(lbm_handle* h, int32_t steps, double* times_ms, int32_t cap, int32_t* n_tried) {
     if (!h || steps < 1) return LBM_EINVAL;
     if (!h->initialised) return LBM_ESTATE;

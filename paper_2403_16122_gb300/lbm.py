@@ -72,7 +72,7 @@ SYMBOLS = (
     "lbm_step_count", "lbm_launch_count", "lbm_destroy", "lbm_error_string",
     "lbm_set_kernel", "lbm_get_kernel", "lbm_autotune", "lbm_step_noalloc",
     "lbm_set_exec", "lbm_get_exec", "lbm_barrier_selftest", "lbm_set_thermal_walls",
-    "lbm_freezing", "lbm_solid_profile",
+    "lbm_freezing", "lbm_solid_profile", "lbm_get_step_kernel",
 )
 LBM_KERNEL_TILE, LBM_KERNEL_STRIP, LBM_KERNEL_STAGED, LBM_KERNEL_BLOCK = 0, 1, 2, 3
 LBM_EXEC_LAUNCH, LBM_EXEC_GRAPH, LBM_EXEC_PERSISTENT = 0, 1, 2
@@ -110,6 +110,8 @@ def load(path: str | None = None):
         lib.lbm_set_kernel.restype = ctypes.c_int
         lib.lbm_get_kernel.argtypes = [vp, P(i32)]
         lib.lbm_get_kernel.restype = ctypes.c_int
+        lib.lbm_get_step_kernel.argtypes = [vp, P(i32)]
+        lib.lbm_get_step_kernel.restype = ctypes.c_int
         lib.lbm_autotune.argtypes = [vp, i32, dp, i32, P(i32)]
         lib.lbm_autotune.restype = ctypes.c_int
         lib.lbm_step_noalloc.argtypes = [P(lbm_params), vp, vp, vp, vp, i32, vp, vp]
@@ -278,6 +280,14 @@ def lbm_get_kernel(h):
     return tuple(out[:])
 
 
+def lbm_get_step_kernel(h):
+    out = (ctypes.c_int32 * 4)()
+    rc = load().lbm_get_step_kernel(h, out)
+    if rc:
+        raise LbmError(rc, "lbm_get_step_kernel")
+    return tuple(out[:])
+
+
 def lbm_set_exec(h, mode: int, chunk: int = 64):
     rc = load().lbm_set_exec(h, int(mode), int(chunk))
     if rc:
@@ -415,6 +425,11 @@ class Lattice:
     @property
     def kernel(self):
         return lbm_get_kernel(self._h)
+
+    @property
+    def step_kernel(self):
+        """The layout that step() runs in now (kernel: the one chosen)."""
+        return lbm_get_step_kernel(self._h)
 
     @property
     def step_count(self) -> int:

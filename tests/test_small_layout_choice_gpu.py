@@ -57,3 +57,30 @@ def test_autotuner_keeps_small_16bit_lattices_in_tiles(lbm, storage):
     assert a.kernel == (lbm.LBM_KERNEL_TILE, 32, 4, 0)
     b = _drop(lbm, storage).set_kernel(*a.kernel)
     assert b.kernel == a.kernel
+
+
+@pytest.mark.parametrize("storage", ["FP32", "FP16", "BF16"])
+def test_step_kernel_is_what_runs(lbm, storage):
+    """kernel reports the chosen layout, step_kernel the one that steps: tiles
+    on a small handle as it was created, and only there. Handing it to a second
+    handle gives the same bits; the persistent form and a chosen layout run as
+    they are reported."""
+    a = _drop(lbm, storage)
+    assert a.kernel[0] == lbm.LBM_KERNEL_STAGED
+    assert a.step_kernel == (lbm.LBM_KERNEL_TILE, 32, 4, 0)
+    b = _drop(lbm, storage).set_kernel(*a.step_kernel)
+    assert b.kernel == b.step_kernel == a.step_kernel
+    for u, v in zip(a.step(10).get_state(), b.step(10).get_state()):
+        assert np.array_equal(u, v)
+    a.set_exec(lbm.LBM_EXEC_PERSISTENT, 4)
+    assert a.step_kernel == a.kernel
+    a.set_exec(lbm.LBM_EXEC_LAUNCH)
+    assert a.step_kernel[0] == lbm.LBM_KERNEL_TILE
+    a.set_kernel(lbm.LBM_KERNEL_STAGED, 4, 0, 168)
+    assert a.step_kernel == a.kernel
+    big = _drop(lbm, storage, 512)
+    assert big.step_kernel == big.kernel and big.kernel[0] == lbm.LBM_KERNEL_STAGED
+    p, _, _ = inputs.stefan(nx=64)  # walls in x
+    if storage == "FP32":
+        lat = lbm.Lattice([p])
+        assert lat.step_kernel == lat.kernel == (lbm.LBM_KERNEL_TILE, 32, 4, 0)

@@ -2660,7 +2660,7 @@ cudaError_t StripPart<ST, STAGED>::persist_launch(int warps, int regs, int grid,
 }
 #endif
 
-#if LBM_PART == 1
+#if LBM_HAS_PART(1)
 namespace {
 constexpr int kNoW = 4, kNoMinB = 3, kNoStg = 3;  // the handles' default variant
 constexpr int kNoSmem = kNoW * warp_smem_floats<float, kNoStg>() * (int)sizeof(float);
@@ -2691,6 +2691,11 @@ cudaError_t launch_step_noalloc_strip(const Inst& I, int rows, int n_items, doub
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, step_strip_noalloc<kNoW, kNoMinB, kNoStg>, I, rows, n_items, scratch);
 }
+#endif
+
+// The strip kernels of a part (in a whole-file compilation their uses
+// instantiate them).
+#if LBM_PART == 1
 template struct StripPart<float, true>;
 #elif LBM_PART == 2
 template struct StripPart<float, false>;

@@ -62,3 +62,19 @@ def test_no_read_only_loads_of_data_still_being_written():
         ["row + p0 + 32 * k) : 0.0"]
     assert "ld_live(row + p0 + 32 * k)" in kern
     assert "ld_live(p + (c + 8 * k) * stride)" in _body(red, "sum_values")
+
+
+def test_whole_file_compilation_defines_every_entry():
+    """lbm_kernels.cu compiled without LBM_PART holds every part: each function
+    that lbm_internal.h declares is defined by it or by another source."""
+    import subprocess
+
+    cmd = [lbm_build.nvcc(), *lbm_build.ARCH, "-std=c++17", f"-I{lbm_build.INCLUDE}",
+           f"-I{lbm_build.CSRC}", "-E", os.path.join(lbm_build.CSRC, "lbm_kernels.cu")]
+    txt = subprocess.run(cmd, capture_output=True, text=True, check=True).stdout
+    txt += _code("lbm_api.cu")
+    header = _code("lbm_internal.h")
+    names = re.findall(r"^(?:cudaError_t|int|bool|void) (\w+)\([^{};]*\);", header, flags=re.M)
+    assert len(names) >= 20 and "launch_step_noalloc_strip" in names
+    missing = [n for n in names if not re.search(r"\b%s\([^{};]*\)\s*\{" % n, txt)]
+    assert missing == []

@@ -341,7 +341,7 @@ cudaError_t launch_init(const Inst* d_inst, int inst, int n_sites, int storage,
 // State transfer of one lattice in FP32 storage, two planes of n_sites doubles
 // at a time (plane q: population q of 27, then carried field q - 27; L the
 // latent heat): planes q0 .. q0 + n_q - 1 out of the buffer, or planes qa and
-// qb (none: -1) into it; plane 9 (h_0) goes in together with plane 27 (f_l).
+// qb (both) into it; plane 9 (h_0) goes in together with plane 27 (f_l).
 cudaError_t launch_planes_from_state(const Inst* d_inst, int inst, int n_sites, int parity, double L,
                                      int q0, int n_q, double* d_out, cudaStream_t s);
 cudaError_t launch_state_from_planes(const Inst* d_inst, int inst, int n_sites, int parity, double L,

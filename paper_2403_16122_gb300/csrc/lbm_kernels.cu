@@ -952,7 +952,7 @@ __device__ __forceinline__ void split_gh(const typename Raw<ST>::Pair raw[9], co
 // thread, and the second block barrier is met only by tiles at a wall. The
 // ring sites' walls, corners and the two extra cells a wall row needs beyond
 // the ring are the same entries for every step. `I` is read from shared memory.
-// The tile's mdot is left in s_md (one value a warp; the caller synchronises
+// The tile's mdot is left in sh.md (one value a warp; the caller synchronises
 // and adds them up).
 template <int TX, int TY, typename ST = float>
 struct TileShared {
@@ -963,7 +963,6 @@ struct TileShared {
     float md[TX * TY / 32];
     float col[TY][TX];                              // f_s (observable steps)
     Inst inst;
-    int ok;
 };
 // What a thread of a tile does in every step, worked out once per launch: its
 // own site and the ring entry it serves, with the offsets of their loads.
@@ -1576,8 +1575,8 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
                                            float* ring = nullptr) {
     constexpr bool kHalf = sizeof(ST) != 4;
     static_assert(STG == 0 || STG >= 3, "staging needs at least three ring slots");
-    // Staging: the collision reads its populations from the ring slot (FP16:
-    // g, h decoded over the staged words; f decoded into registers)
+    // Staging: the collision reads its populations from the ring slot (16-bit
+    // storage: g and h decoded there once more, f decoded into registers)
     constexpr bool kSlotPops = STG > 0;
     const int lane = threadIdx.x & 31;
     const Inst& I = insts[W.inst];

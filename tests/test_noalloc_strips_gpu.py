@@ -1,8 +1,9 @@
-"""lbm_step_noalloc in staged strips (lattices periodic in x of more than two
-waves of tiles) against the tile kernel of a handle, on the same state."""
+"""lbm_step_noalloc in strips (lattices periodic in x of more than two waves of
+tiles) and in tiles against another tile kernel of a handle, on the same state,
+every column of it."""
 import numpy as np
 import pytest
-from test_zz_no_alloc import _blocked
+from test_zz_no_alloc import _blocked, _unblocked
 
 from paper_2403_16122_gb300 import inputs
 
@@ -51,3 +52,36 @@ def test_record_is_summed_in_64_bits(env, nx, ny):
     assert want["solid"] == got["solid"] == 0.0
     for k in ("volume", "enthalpy"):
         assert got[k] == pytest.approx(want[k], rel=1e-13), k
+
+
+# strips (whole and ragged last strips, a pitch wider than they need), then
+# tiles: two waves at most, walls in x, more 32 x 4 tiles than partial slots
+LAYOUTS = [(500, 420, 1, 512), (500, 420, 1, 576), (512, 512, 1, 512), (1501, 131, 1, 1568),
+           (483, 430, 1, 512), (100, 90, 1, 128), (450, 400, 0, 480), (1000, 1100, 0, 1024)]
+
+
+@pytest.mark.parametrize("nx,ny,px,pitch", LAYOUTS)
+def test_every_column_matches_other_tiles(env, nx, ny, px, pitch):
+    """Two steps against a handle in 64 x 4 tiles, which no allocation-free step
+    uses: layouts agree within 1e-6, in every column, the ragged last strip and
+    the wall columns included, and the padding is never written."""
+    torch, lbm = env
+    p = inputs.params(nx=nx, ny=ny, periodic_x=px, periodic_y=0, dirichlet_y_lo=1,
+                      dirichlet_y_hi=ny % 2, dirichlet_x_hi=1 - px, theta_deg=60.0)
+    phi0, T0 = inputs.random_state(p, seed=nx + pitch)
+    L = p["Cp"] * (p["T_m"] - p["T_w"]) / p["Ste"]
+    lat = lbm.Lattice([p]).set_kernel(lbm.LBM_KERNEL_TILE, 64, 4).init(phi0, T0).step(2)
+    for call in range(2):
+        pops, aux = lat.get_state()
+        want = lat.step(1)
+        Po, Ao, rec = _noalloc_step(env, p, pops, aux, pitch)
+        got = _unblocked(Po, Ao, L, nx, ny, pitch)
+        for a, b in zip(got, want.get_state()):
+            assert np.abs(a - b).max() <= 1e-6, call
+        pad = Po.reshape(ny, pitch // 32, 768)[:, (nx + 31) // 32:]
+        assert not pad.any()
+        obs = want.observables(check=False)
+        for k in ("volume", "solid", "enthalpy", "mass", "condensed_mass", "solid_col", "solid_row"):
+            assert rec[k] == pytest.approx(obs[k], rel=1e-6, abs=1e-6), (call, k)
+        assert rec["umax"] == pytest.approx(obs["umax"], rel=1e-3, abs=1e-6)
+    lat.close()

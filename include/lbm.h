@@ -331,9 +331,12 @@ int lbm_autotune(lbm_handle* h, int32_t steps, double* times_ms, int32_t cap, in
 #define LBM_EXEC_PERSISTENT  2
 
 /* Select the execution form; chunk in [1, 65536] steps. Captured graphs are
-   dropped (also by lbm_set_kernel, whose tables they use). LBM_EINVAL for an
-   unknown mode or chunk, or PERSISTENT with the tile layout (and
-   lbm_set_kernel refuses the tile layout while PERSISTENT is selected). */
+   dropped (also by lbm_set_kernel, whose tables they use). To or from PERSISTENT
+   on a handle that lbm_create's choice steps in tiles the tables are rebuilt,
+   which synchronises the stream (LBM_ECUDA while it is being captured; the form
+   stays as it was). LBM_EINVAL for an unknown mode or chunk, or PERSISTENT with
+   the tile layout (and lbm_set_kernel refuses the tile layout while PERSISTENT
+   is selected). */
 int lbm_set_exec(lbm_handle* h, int32_t mode, int32_t chunk);
 
 /* out[0] = mode, out[1] = chunk, out[2] = CTAs of one persistent launch for

@@ -168,6 +168,7 @@ struct lbm_handle {
     int tx = kTileX, ty = kTileY;        // tile shape
     bool chosen = true;                  // the layout is still the one lbm_create chose
     bool small = false;                  // all lattices together: two waves of tiles at most
+    bool tables_ok = false;              // host and device tables are those of the layout
     int warps = 4, rows = 16, regs = 168; // strip layouts (rows: effective)
     int rows_req = 16;                    // requested rows per item, 0 = one wave
     std::vector<Item> items;
@@ -220,8 +221,11 @@ struct lbm_handle {
 
 namespace {
 
+// Code of a failed call. The error is reported here: cleared, so that the check
+// after a later launch does not find it.
 int cuda_fail(cudaError_t e) {
     (void)e;
+    cudaGetLastError();
     return LBM_ECUDA;
 }
 
@@ -476,7 +480,9 @@ int restart_records(lbm_handle* h, int k) {
     return LBM_OK;
 }
 
+// (a failure leaves tables_ok down, and the next step rebuilds them first)
 int upload_tables(lbm_handle* h) {
+    h->tables_ok = false;
     drop_graphs(h);  // captured launches carry the old item counts
     {
         const int rc = fold_mdot(h);
@@ -515,6 +521,7 @@ int upload_tables(lbm_handle* h) {
                                  ? lbmk::persistent_grid(h->kind == LBM_KERNEL_STAGED, h->warps,
                                                          h->regs, h->storage, items_at(h, h->rows))
                                  : 0);
+    h->tables_ok = true;
     return LBM_OK;
 }
 
@@ -760,6 +767,10 @@ int lbm_step(lbm_handle* h, int64_t n) {
     if (!h || n < 0) return LBM_EINVAL;
     if (!h->initialised) return LBM_ESTATE;
     if (h->failed) return LBM_ETIMEOUT;
+    if (!h->tables_ok) {
+        const int rc = upload_tables(h);
+        if (rc != LBM_OK) return rc;
+    }
     h->clock += n;
     if (h->kind == LBM_KERNEL_BLOCK && n > 0) h->persist_pending = true;  // its error word too
     // every step but the last runs without observables, in the handle's form
@@ -1136,9 +1147,16 @@ int lbm_set_exec(lbm_handle* h, int32_t mode, int32_t chunk) {
         return LBM_EINVAL;
     drop_graphs(h);
     const bool was_tiled = tiled(h);
+    const int old_mode = h->exec, old_chunk = h->chunk;
     h->exec = mode;
     h->chunk = chunk;
-    return tiled(h) == was_tiled ? LBM_OK : upload_tables(h);
+    if (tiled(h) == was_tiled) return LBM_OK;
+    const int rc = upload_tables(h);
+    if (rc != LBM_OK) {  // as it was (the tables are rebuilt before the next step)
+        h->exec = old_mode;
+        h->chunk = old_chunk;
+    }
+    return rc;
 }
 
 int lbm_get_exec(const lbm_handle* h, int32_t* out) {

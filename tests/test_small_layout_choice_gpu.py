@@ -84,3 +84,33 @@ def test_step_kernel_is_what_runs(lbm, storage):
     if storage == "FP32":
         lat = lbm.Lattice([p])
         assert lat.step_kernel == lat.kernel == (lbm.LBM_KERNEL_TILE, 32, 4, 0)
+
+
+def test_failed_change_of_form_leaves_the_handle_as_it_was(lbm):
+    """To the persistent form a small handle rebuilds its tables, which waits for
+    the stream: an error while the stream is being captured. The handle then
+    steps on as before, on the same tables."""
+    import ctypes
+
+    import torch
+
+    s = torch.cuda.Stream()
+    p, phi0, T0 = inputs.sessile(nx=96, ny=64, R=24.0)
+    a, b = (lbm.Lattice([p], stream=s).init(phi0, T0).step(3) for _ in range(2))
+    cu = ctypes.CDLL("libcuda.so.1")
+    stream, graph = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
+    torch.cuda.synchronize()
+    assert cu.cuStreamBeginCapture_v2(stream, 1) == 0  # of this thread
+    with pytest.raises(lbm.LbmError) as e:
+        a.set_exec(lbm.LBM_EXEC_PERSISTENT, 4)
+    assert e.value.code == lbm.LBM_ECUDA
+    assert cu.cuStreamEndCapture(stream, ctypes.byref(graph)) != 0  # the capture is void
+    assert a.exec[:2] == b.exec[:2] and a.step_kernel == b.step_kernel
+    for u, v in zip(a.step(20).get_state(), b.step(20).get_state()):
+        assert np.array_equal(u, v)
+    assert a.observables() == b.observables()
+    assert a.freezing() == b.freezing()
+    a.set_exec(lbm.LBM_EXEC_PERSISTENT, 4)
+    assert a.step_kernel[0] == lbm.LBM_KERNEL_STAGED
+    a.step(9)
+    assert a.observables()["nonfinite"] == 0.0

@@ -1045,7 +1045,9 @@ int get_state_fp32(lbm_handle* h, int32_t inst, double* pops, double* aux) {
     };
     cudaError_t e = pops ? planes(0, 27, pops) : cudaSuccess;
     if (e == cudaSuccess && aux) e = planes(27, 32, aux);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    // also after a failure: no copy to the caller's arrays outlives the call
+    const cudaError_t done = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = done;
     return e == cudaSuccess ? LBM_OK : cuda_fail(e);
 }
 
@@ -1053,11 +1055,11 @@ int set_state_fp32(lbm_handle* h, int32_t inst, const double* pops, const double
     const size_t n = (size_t)h->params[inst].nx * h->params[inst].ny;
     auto plane = [&](int q) { return q < 27 ? pops + (size_t)q * n : aux + (size_t)(q - 27) * n; };
     // every plane once: h_0 with f_l, which its shift needs, the others in pairs
-    std::vector<int> order = {9, 27};
+    int order[32] = {9, 27}, n_order = 2;
     for (int q = 0; q < 32; ++q)
-        if (q != 9 && q != 27) order.push_back(q);
+        if (q != 9 && q != 27) order[n_order++] = q;
     cudaError_t e = cudaSuccess;
-    for (size_t a = 0; a < order.size() && e == cudaSuccess; a += 2) {
+    for (int a = 0; a < 32 && e == cudaSuccess; a += 2) {
         for (int b = 0; b < 2 && e == cudaSuccess; ++b)
             e = cudaMemcpyAsync(h->d_stage + b * n, plane(order[a + b]), n * sizeof(double),
                                 cudaMemcpyHostToDevice, h->stream);
@@ -1065,7 +1067,9 @@ int set_state_fp32(lbm_handle* h, int32_t inst, const double* pops, const double
             e = lbmk::launch_state_from_planes(h->d_inst, inst, (int)n, h->parity, h->init_L[inst],
                                                order[a], order[a + 1], h->d_stage, h->stream);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // the caller's arrays are read
+    // also after a failure: no copy from the caller's arrays outlives the call
+    const cudaError_t done = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = done;
     if (e != cudaSuccess) return cuda_fail(e);
     h->initialised = true;
     h->have_obs = false;

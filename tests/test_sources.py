@@ -78,3 +78,18 @@ def test_whole_file_compilation_defines_every_entry():
     assert len(names) >= 20 and "launch_step_noalloc_strip" in names
     missing = [n for n in names if not re.search(r"\b%s\([^{};]*\)\s*\{" % n, txt)]
     assert missing == []
+
+
+def test_state_transfer_waits_for_its_copies_after_a_failure_too():
+    """lbm_get_state and lbm_set_state in FP32 storage copy plane by plane between
+    the device and the caller's arrays, which may be pinned: copies queued before
+    a call that fails still run. The stream is waited for on every way out."""
+    api = _code("lbm_api.cu")
+    for name in ("get_state_fp32", "set_state_fp32"):
+        body = _body(api, name)
+        wait = body.index("cudaStreamSynchronize")
+        # unconditional, and no way out of the function before it
+        assert re.search(r"\n    const cudaError_t \w+ = cudaStreamSynchronize", body), name
+        outer = re.sub(r"auto (planes|plane) = \[&\].*?\n    \};|auto plane = [^;]*;[^;]*;",
+                       "", body[:wait], flags=re.S)
+        assert "return" not in outer, name

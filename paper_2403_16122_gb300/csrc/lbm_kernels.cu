@@ -425,23 +425,25 @@ struct SiteObs {
         }
     }
     __device__ __forceinline__ void max(int j, float x) { v[j] = x; }
-    __device__ __forceinline__ float greatest() const { return v[9]; }
-    __device__ __forceinline__ bool some(int j) const { return v[j] != 0.f; }
     __device__ __forceinline__ double total(int j) const {
         return j == 2 ? (double)v[2] + ((double)h[0] + (double)h[1]) : (double)v[j];
     }
 };
 
-// FP64 totals of a warp's lanes, handed to put(j, total) by one lane each.
-// Slots 0-6 go through one reduce-scatter: at lane bits 4, 3 and 2 a lane keeps
-// half of its vector and adds the partner's copy of that half, then two xor
-// steps finish, so a warp issues 9 FP64 additions for them instead of 35 (FP64
-// runs at two additions a cycle and SM here: eleven plain trees were 3.5 us of
-// the tiles' observable step). Slot 9 is a maximum of FP32 values; slots 7, 8
-// and 10 are zero but for a few sites and are skipped where a warp has none.
-template <typename Acc, typename Put>
-__device__ __forceinline__ void warp_totals(const Acc& ob, int lane, Put&& put) {
+// Block reduction of the observables of a tile (FP64). out: the tile's slot in
+// observable-major partials (observable j at out[j * stride]). A warp's sums of
+// slots 0-6 go through one reduce-scatter: at lane bits 4, 3 and 2 a lane
+// keeps half of its vector and adds the partner's copy of that half, then two
+// xor steps finish, so a warp issues 9 FP64 additions for them instead of 35
+// (FP64 runs at two additions a cycle and SM here: eleven plain trees were
+// 3.5 us of the observable step). Slot 9 is a maximum of FP32 values; slots 7,
+// 8 and 10 are zero but for a few sites and are skipped where a warp has none.
+template <int NT>
+__device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __restrict__ out,
+                                                 int stride) {
+    __shared__ double red[NT / 32][kObs];
     constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
     double k4[4], k2[2];
 #pragma unroll
@@ -455,33 +457,23 @@ __device__ __forceinline__ void warp_totals(const Acc& ob, int lane, Put&& put) 
     double t = (b2 ? k2[1] : k2[0]) + __shfl_xor_sync(kAll, b2 ? k2[0] : k2[1], 4);
     t += __shfl_xor_sync(kAll, t, 2);
     t += __shfl_xor_sync(kAll, t, 1);
-    if ((lane & 3) == 0 && lane < 28) put(lane >> 2, t);
-    float mx = ob.greatest();
+    if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
+    float mx = ob.v[9];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kAll, mx, o));
-    if (lane == 0) put(9, (double)mx);
+    if (lane == 0) red[warp][9] = (double)mx;
     auto rare = [&](int j) {
         double x = 0.0;
-        if (__any_sync(kAll, ob.some(j))) {
+        if (__any_sync(kAll, ob.v[j] != 0.f)) {
             x = ob.total(j);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
         }
-        if (lane == 0) put(j, x);
+        if (lane == 0) red[warp][j] = x;
     };
     rare(7);
     rare(8);
     rare(10);
-}
-
-// Block reduction of the observables of a tile (FP64). out: the tile's slot in
-// observable-major partials (observable j at out[j * stride]).
-template <int NT>
-__device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __restrict__ out,
-                                                 int stride) {
-    __shared__ double red[NT / 32][kObs];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    warp_totals(ob, lane, [&](int j, double x) { red[warp][j] = x; });
     __syncthreads();
     if (threadIdx.x < kObs) {
         const int j = threadIdx.x;
@@ -491,43 +483,85 @@ __device__ __forceinline__ void block_reduce_obs(const SiteObs& ob, double* __re
     }
 }
 
-// Observable sums of a strip, lane by lane over an item's rows (the
-// allocation-free step, whose caller reads the record of one step as FP64): a
-// running FP32 sum and the sum of the exact rounding errors of its additions
-// (D. E. Knuth, "The Art of Computer Programming", vol. 2, 4.2.2), so that a
-// lane's sum keeps some 48 bits, then FP64 across the lanes and items: the sum of
-// phi is within 2e-16 of the exact one on 500 x 420 to 1900 x 1000 sites, as the
-// tiles' is. A step of 512 x 512 sites, us: 24.7; FP64 additions row by row
-// 31.3; the rows in FP32 (RowObs below, 1.5e-9) 23.2.
+// An FP32 sum and the sum of the exact rounding errors of its additions (D. E.
+// Knuth, "The Art of Computer Programming", vol. 2, 4.2.2): some 48 bits.
+struct PairSum {
+    float s, c;
+    __device__ __forceinline__ void add(float x, float xc = 0.f) {
+        const float t = s + x, d = t - s;
+        c += ((s - (t - d)) + (x - d)) + xc;
+        s = t;
+    }
+    __device__ __forceinline__ void add_lane(const PairSum& o, int mask) {
+        const float os = __shfl_xor_sync(0xffffffffu, o.s, mask);
+        add(os, __shfl_xor_sync(0xffffffffu, o.c, mask));
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
+// Observable sums of a strip, lane by lane over an item's rows and then across
+// the lanes, in pairs (the allocation-free step, whose caller reads the record
+// of one step as FP64); FP64 across the items. The sum of phi is within 2e-16 of
+// the exact one on 500 x 420 to 1900 x 1000 sites, as the tiles' is. A step of 512
+// x 512 sites, us: 21.9; with FP64 across the lanes 24.5, FP64 row by row 31.3;
+// the rows in FP32 (RowObs below, off by up to 1.5e-9) 22.9.
 struct LaneObs {
-    float s[7], c[7], mx, row, bad;
+    PairSum p[7];
+    float mx, row, bad;
     bool col;
     __device__ __forceinline__ void zero() {
 #pragma unroll
-        for (int j = 0; j < 7; ++j) s[j] = c[j] = 0.f;
+        for (int j = 0; j < 7; ++j) p[j] = PairSum{0.f, 0.f};
         mx = row = bad = 0.f;
         col = false;
     }
     __device__ __forceinline__ void add(int j, float x) {
-        if (j == 7) {  // a lane's column: its sum of f_s, slot 1
-            col = true;
-        } else if (j == 8) {  // one row of the item at most
-            row = x;
-        } else if (j == 10) {
-            bad += x;
-        } else {
-            const float t = s[j] + x, d = t - s[j];
-            c[j] += (s[j] - (t - d)) + (x - d);
-            s[j] = t;
-        }
+        if (j == 7) col = true;      // a lane's column: its sum of f_s, slot 1
+        else if (j == 8) row = x;    // one row of the item at most
+        else if (j == 10) bad += x;
+        else p[j].add(x);
     }
     __device__ __forceinline__ void max(int, float x) { mx = fmaxf(mx, x); }
     __device__ __forceinline__ void flush(int) {}
-    __device__ __forceinline__ float greatest() const { return mx; }
-    __device__ __forceinline__ bool some(int j) const { return j == 7 ? col : (j == 8 ? row != 0.f : bad != 0.f); }
-    __device__ __forceinline__ double total(int j) const {
-        if (j < 7) return (double)s[j] + (double)c[j];
-        return j == 7 ? (col ? total(1) : 0.0) : (double)(j == 8 ? row : bad);
+    // all 32 lanes, once: the reduce-scatter of block_reduce_obs
+    __device__ __forceinline__ void store(int lane, double* out, long long stride) const {
+        constexpr unsigned kAll = 0xffffffffu;
+        const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+        const PairSum none{0.f, 0.f};
+        PairSum k4[4], k2[2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const PairSum lo = p[q], hi = q + 4 < 7 ? p[q + 4] : none;
+            k4[q] = b4 ? hi : lo;
+            k4[q].add_lane(b4 ? lo : hi, 16);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            k2[q] = b3 ? k4[q + 2] : k4[q];
+            k2[q].add_lane(b3 ? k4[q] : k4[q + 2], 8);
+        }
+        PairSum t = b2 ? k2[1] : k2[0];
+        t.add_lane(b2 ? k2[0] : k2[1], 4);
+        t.add_lane(t, 2);
+        t.add_lane(t, 1);
+        float m = mx, n = bad;  // (a count below 2^24: exact)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
+            n += __shfl_xor_sync(kAll, n, o);
+        }
+        PairSum r = none;
+        if (__any_sync(kAll, row != 0.f)) {
+            r.s = row;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) r.add_lane(r, o);
+        }
+        const unsigned at = __ballot_sync(kAll, col);
+        if ((lane & 3) == 0 && lane < 28) out[(lane >> 2) * stride] = t.value();
+        if (lane == (at ? __ffs(at) - 1 : 0)) out[7 * stride] = at ? p[1].value() : 0.0;
+        if (lane == 1) out[8 * stride] = r.value();
+        if (lane == 2) out[9 * stride] = (double)m;
+        if (lane == 3) out[10 * stride] = (double)n;
     }
 };
 
@@ -1874,7 +1908,7 @@ __device__ __forceinline__ void strip_item(const Inst* __restrict__ insts, const
     if constexpr (STG > 0) cp_async_wait<0>();  // the trailing groups are empty
 
     if constexpr (std::is_same_v<Obs, LaneObs>) {
-        warp_totals(ob, lane, [&](int j, double x) { partials[(long long)j * I.part_stride + W.part] = x; });
+        ob.store(lane, partials + W.part, I.part_stride);
     } else {
         if (OBS && RowObs::carried(lane) >= 0)
             partials[(long long)RowObs::carried(lane) * I.part_stride + W.part] = ob.total();

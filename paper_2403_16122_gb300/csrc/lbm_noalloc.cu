@@ -87,7 +87,7 @@ extern "C" int lbm_step_noalloc(const lbm_params* p, const float* pops_in, const
     // Layout as lbm_create chooses it: 32 x 4 tiles while they are two waves or
     // less (four steps: 67 us on 256 x 256 sites, 136 us in the 32 x 8 tiles of
     // before), else strips in one wave where the lattice is periodic in x (512 x
-    // 512: 99 us against 172 in tiles), else tiles, 32 x 8 where the shorter ones
+    // 512: 91 us against 172 in tiles), else tiles, 32 x 8 where the shorter ones
     // are more than the LBM_NOALLOC_MAX_TILES slots (closed 512 x 512: 146 us in
     // 32 x 8, 363 before).
     const long long small_tiles = (long long)tiles_x * ((p->ny + 3) / 4);

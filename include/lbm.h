@@ -265,7 +265,8 @@ int lbm_set_state(lbm_handle* h, int32_t inst, const double* pops,
    waves of 32 x 4 tiles or less (some 155,000 sites) are stepped by
    the tile kernel, where one step of so few sites is shorter; the persistent
    execution form, and a layout chosen by lbm_set_kernel or lbm_autotune, run
-   as they are reported. */
+   as they are reported. A lattice alone and the same lattice in a larger batch
+   may so run in different layouts and agree to rounding. */
 #define LBM_KERNEL_TILE   0
 #define LBM_KERNEL_STRIP  1
 #define LBM_KERNEL_STAGED 2
